@@ -181,15 +181,19 @@ struct ConvGeom {
   }
 };
 
-// Optional work of a forward convolution's epilogue (nullptr = off):
+// Optional work of a convolution's epilogue (nullptr = off), forward unless
+// noted:
 //   pool  the 2x2x2 mean of the (bf16-rounded) outputs on the D/2 grid,
 //         N <= 32 and ZB even (both z slices of a pair are in the thread,
 //         the x / y partners are lanes ^1 / ^8 of the warp);
+//   mask  (input gradient) activations [B][D^3][N]: the ReLU derivative, the
+//         gradient is written as 0 where they are not above 0;
 //   hw    the linear head (N = 16): delta = hb + sum_c out_c hw_c,
 //         pred = base + norm[3 sample + 2] delta (float fields [B][D^3]);
 //         with store_out = 0 the activations themselves are not written.
 struct ConvEpi {
   __nv_bfloat16 *pool = nullptr;
+  const __nv_bfloat16 *mask = nullptr;
   const float *hw = nullptr, *base = nullptr, *norm = nullptr;
   float *delta = nullptr, *pred = nullptr;
   int store_out = 1;
@@ -390,7 +394,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __nv_bfloat16
               float dlt = __ldg(ep.hw + 16);  // the head's bias
 #pragma unroll
               for (int c = 0; c < 16; ++c) dlt = fmaf(v[c], __ldg(ep.hw + c), dlt);
-              ep.delta[vox] = dlt;
+              if (ep.delta) ep.delta[vox] = dlt;
               if (ep.pred) ep.pred[vox] = ep.base[vox] + ep.norm[3 * sample + 2] * dlt;
             }
             if (ep.pool != nullptr) {
@@ -435,11 +439,20 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __nv_bfloat16
         for (int g = 0; g < 2; ++g) {
           if (g >= ng) break;
           const int col = col0 + 16 * g, zz = col / N, c0 = col % N;
-          __nv_bfloat16 *dst = out + (vbase + (int64_t)(bz * ZB + zz) * D * D) * N + c0;
-          __align__(16) __nv_bfloat162 o[8];
+          const int64_t at = (vbase + (int64_t)(bz * ZB + zz) * D * D) * N + c0;
+          __nv_bfloat16 *dst = out + at;
+          __align__(16) __nv_bfloat162 o[8], act[8];
+          if (!FWD && ep.mask != nullptr) {
+            reinterpret_cast<uint4 *>(act)[0] = __ldg(reinterpret_cast<const uint4 *>(ep.mask + at));
+            reinterpret_cast<uint4 *>(act)[1] = __ldg(reinterpret_cast<const uint4 *>(ep.mask + at) + 1);
+          }
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             float a = v[16 * g + 2 * q], b2 = v[16 * g + 2 * q + 1];
+            if (!FWD && ep.mask != nullptr) {
+              if (!(__low2float(act[q]) > 0.f)) a = 0.f;
+              if (!(__high2float(act[q]) > 0.f)) b2 = 0.f;
+            }
             if (FWD) {
               a = fmaxf(a + __ldg(bias + c0 + 2 * q), 0.f);
               b2 = fmaxf(b2 + __ldg(bias + c0 + 2 * q + 1), 0.f);
@@ -507,31 +520,18 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_tc(const __nv_bfloat16
   if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(G::kCols));
 }
 
-// Weight images for k_conv_tc from src [N][27][K] (bf16):
+// Place of weight (n, t, k) in the weight image of k_conv_tc<N, ...>:
 //   per tap (N >= 48):  [K/16][27 taps][2 K-halves][N][8]
 //   stacked (N <= 32):  [K/16][9 (dy, dx)][2 K-halves][3 (dz = +1, 0, -1)][N][8]
 // with the tap offsets of the stacked form scaled by `sign` (-1 for the
 // input-gradient convolution, whose taps are mirrored).
-__global__ void k_weight_image(const __nv_bfloat16 *__restrict__ src, int N, int K, int sign,
-                               __nv_bfloat16 *__restrict__ dst) {
-  const int64_t total = (int64_t)N * 27 * K;
-  const bool stack = N <= 32;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int k = (int)(e % K);
-    const int t = (int)((e / K) % 27);
-    const int n = (int)(e / (27 * K));
-    const int kc = k >> 4, p = (k >> 3) & 1, j = k & 7;
-    int64_t o;
-    if (!stack) {
-      o = ((((int64_t)kc * 27 + t) * 2 + p) * N + n) * 8 + j;
-    } else {
-      // applied offsets (dzs, dys, dxs) = sign (dz, dy, dx) of tap t
-      const int dzs = sign * (t / 9 - 1), dys = sign * ((t / 3) % 3 - 1), dxs = sign * (t % 3 - 1);
-      const int q = (dys + 1) * 3 + (dxs + 1), st = 1 - dzs;  // dzs = +1 -> 0, 0 -> 1, -1 -> 2
-      o = (((((int64_t)kc * 9 + q) * 2 + p) * 3 + st) * N + n) * 8 + j;
-    }
-    dst[o] = src[e];
-  }
+__device__ __forceinline__ int image_index(int N, int sign, int n, int t, int k) {
+  const int kc = k >> 4, p = (k >> 3) & 1, j = k & 7;
+  if (N > 32) return (((kc * 27 + t) * 2 + p) * N + n) * 8 + j;
+  // applied offsets (dzs, dys, dxs) = sign (dz, dy, dx) of tap t
+  const int dzs = sign * (t / 9 - 1), dys = sign * ((t / 3) % 3 - 1), dxs = sign * (t % 3 - 1);
+  const int q = (dys + 1) * 3 + (dxs + 1), st = 1 - dzs;  // dzs = +1 -> 0, 0 -> 1, -1 -> 2
+  return ((((kc * 9 + q) * 2 + p) * 3 + st) * N + n) * 8 + j;
 }
 
 }  // namespace tc

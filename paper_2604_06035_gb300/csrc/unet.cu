@@ -68,7 +68,8 @@ __device__ __forceinline__ int64_t halo_row(int64_t sbase, int D, int bz, int by
 // (in = output gradient, W = [Cin][27][Cout]).  N = 8 NT output channels.
 template <int NT, int SIGN, bool BIAS_RELU>
 __global__ void __launch_bounds__(kConvThreads) k_conv(const bf16 *__restrict__ in, int K, const bf16 *__restrict__ W,
-                                                      const float *__restrict__ bias, bf16 *__restrict__ out, int D) {
+                                                      const float *__restrict__ bias, const bf16 *__restrict__ mask,
+                                                      bf16 *__restrict__ out, int D) {
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int N = NT * 8;
   bf16 *halo = reinterpret_cast<bf16 *>(smem);  // [216][16]
@@ -132,100 +133,183 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(const bf16 *__restrict__ 
       if (BIAS_RELU) {
         x0 = fmaxf(x0, 0.f);
         x1 = fmaxf(x1, 0.f);
+      } else if (mask != nullptr) {  // ReLU derivative from the stored activations
+        const __nv_bfloat162 act = *reinterpret_cast<const __nv_bfloat162 *>(mask + v * N + c0);
+        if (!(__low2float(act) > 0.f)) x0 = 0.f;
+        if (!(__high2float(act) > 0.f)) x1 = 0.f;
       }
       *reinterpret_cast<__nv_bfloat162 *>(out + v * N + c0) = __floats2bfloat162_rn(x0, x1);
     }
   }
 }
 
-// dW[co][t][ci] += sum_v dout[v][co] * in[v + d_t][ci] over the bricks of
-// this block, for the TG taps t0 = TG blockIdx.y ... t0 + TG - 1: each
-// brick's 6x6x6 halo and output gradient are staged once and serve all TG
-// taps.  A tile is (tap, 16 output channels, 16 input channels): two
-// m16n8k16 accumulators; tiles go round-robin to the 8 warps.
-constexpr int kWgThreads = 256;
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 
-template <int CIN, int COUT, int TG>
-__global__ void __launch_bounds__(kWgThreads) k_conv_wgrad(const bf16 *__restrict__ dout, const bf16 *__restrict__ in,
-                                                          float *__restrict__ dW, int D, int nbricks,
-                                                          int bricks_per_block) {
-  constexpr int NMB = COUT / 16, NJP = CIN / 16, TILES = TG * NMB * NJP, MAXT = (TILES + 7) / 8;
+// Weight and bias gradients of one layer:
+//   dW[co][t][ci] += sum_v dout[v][co] in[v + d_t][ci],  db[co] += sum_v dout[v][co].
+// `in` is a tensor of CIN channels, or (up) the channel concatenation of the
+// nearest-upsampled `in` (Ca channels on the D/2 grid) and `skip` (Cb), read
+// in place.
+//
+// What bounds it: with 16 output channels every B fragment (16 voxels x 16
+// input channels, one ldmatrix.x4) feeds only two MMAs, so the ldmatrix reads
+// of shared memory (4 clocks each) weigh as much as the MMAs.  Hence the
+// split: blockIdx.y takes one slice of 16 input channels and all 27 taps, so
+// that a brick's halo is staged once for all of them; a warp takes the 9 taps
+// of one dz and NM tiles of 16 output channels, so that its A fragment
+// (dout^T) is read once for 9 taps and its B fragments serve NM tiles; the
+// warps left over split the brick's voxels (KW ways).  Halo and dout are kept
+// as planes of 8 channels (16-byte rows): 8 consecutive voxels are 128
+// contiguous bytes, conflict-free for ldmatrix, and a tap's offset is an
+// immediate.  Bricks are double-buffered with cp.async; one block per SM
+// walks them and its partial sums are combined in shared memory before one
+// red.v2 per pair of weights.  The bias gradient is one more MMA per A
+// fragment, against ones.
+template <int COUT, int BX, int BY, int BZ>
+struct WgradGeom {
+  static constexpr int kThreads = 384, kWarps = 12;
+  static constexpr int NM = COUT == 16 ? 1 : 2;       // output-channel tiles per warp
+  static constexpr int kGroups = 3 * (COUT / 16 / NM);  // (dz, tile group)
+  static constexpr int KW = kWarps / kGroups;
+  static constexpr int HX = BX + 2, HY = BY + 2, HZ = BZ + 2, kRows = HX * HY * HZ, kVox = BX * BY * BZ;
+  // plane strides: 8 lanes of a copy (8 / planes voxels x planes) hit distinct banks
+  static constexpr int kHaloPlane = (kRows * 16 + 127) / 128 * 128 + 64;
+  static constexpr int kDoutPlane = kVox * 16 + 1024 / COUT;
+  static constexpr int kStage = (2 * kHaloPlane + (COUT / 8) * kDoutPlane + 127) / 128 * 128;
+  static constexpr int kRed = 27 * 16 * COUT * 4;
+  static constexpr int kSmem = 2 * kStage > kRed ? 2 * kStage : kRed;
+};
+
+template <int COUT, int BX, int BY, int BZ>
+__global__ void __launch_bounds__(384, 1) k_conv_wgrad(const bf16 *__restrict__ dout, const bf16 *__restrict__ in,
+                                                      int CIN, const bf16 *__restrict__ skip, int Cb,
+                                                      float *__restrict__ dW, float *__restrict__ db, int D,
+                                                      int nbricks) {
+  using G = WgradGeom<COUT, BX, BY, BZ>;
+  constexpr int NM = G::NM;
   extern __shared__ __align__(16) uint8_t smem[];
-  bf16 *halo = reinterpret_cast<bf16 *>(smem);  // [216][CIN]
-  bf16 *dt = halo + 216 * CIN;                  // [64][COUT]
-  const int t0 = blockIdx.y * TG;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float acc[MAXT][2][4];
-#pragma unroll
-  for (int i = 0; i < MAXT; ++i)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) acc[i][h][0] = acc[i][h][1] = acc[i][h][2] = acc[i][h][3] = 0.f;
-  const int D4 = D >> 2, per = D4 * D4 * D4;
-  const int b_first = blockIdx.x * bricks_per_block;
-  for (int bi = b_first; bi < b_first + bricks_per_block && bi < nbricks; ++bi) {
+  const int group = warp % G::kGroups, kw = warp / G::kGroups;
+  const int dz = group % 3, mb0 = (group / 3) * NM;
+  const int nbx = D / BX, nby = D / BY, per = nbx * nby * (D / BZ);
+  // this block's slice of 16 input channels
+  const int Ca = CIN - Cb, c_first = blockIdx.y * 16;
+  const bool two = skip != nullptr, up = two && c_first < Ca;
+  const bf16 *src = (two && !up) ? skip : in;
+  const int cstride = up ? Ca : (two ? Cb : CIN), cbase = (two && !up) ? c_first - Ca : c_first;
+  const int Dg = up ? D >> 1 : D, sh = up ? 1 : 0;
+
+  auto stage = [&](int bi, int buf) {
     const int s = bi / per, brick = bi % per;
-    const int bx = brick % D4, by = (brick / D4) % D4, bz = brick / (D4 * D4);
-    const int64_t sbase = (int64_t)s * D * D * D;
-    for (int p = threadIdx.x; p < 216 * (CIN / 8); p += kWgThreads) {
-      const int row = p / (CIN / 8), piece = p % (CIN / 8);
-      const int hz = row / 36, hy = (row / 6) % 6, hx = row % 6;
-      const int64_t g = halo_row(sbase, D, bz, by, bx, hz, hy, hx);
-      *reinterpret_cast<uint4 *>(halo + row * CIN + piece * 8) =
-          *reinterpret_cast<const uint4 *>(in + g * CIN + piece * 8);
+    const int x0 = (brick % nbx) * BX, y0 = ((brick / nbx) % nby) * BY, z0 = (brick / (nbx * nby)) * BZ;
+    const uint32_t halo = smem_u32(smem + buf * G::kStage), dt = halo + 2 * G::kHaloPlane;
+    const bf16 *ss = src + (int64_t)s * Dg * Dg * Dg * cstride + cbase;
+    for (int p = threadIdx.x; p < 2 * G::kRows; p += G::kThreads) {
+      const int row = p >> 1, half = p & 1;
+      const int x = wrap(x0 + row % G::HX - 1, D) >> sh, y = wrap(y0 + (row / G::HX) % G::HY - 1, D) >> sh,
+                z = wrap(z0 + row / (G::HX * G::HY) - 1, D) >> sh;
+      cp_async16(halo + half * G::kHaloPlane + row * 16, ss + (((int64_t)z * Dg + y) * Dg + x) * cstride + half * 8);
     }
-    for (int p = threadIdx.x; p < 64 * (COUT / 8); p += kWgThreads) {
-      const int vi = p / (COUT / 8), piece = p % (COUT / 8);
-      const int64_t v = sbase + ((int64_t)(bz * 4 + vi / 16) * D + by * 4 + (vi / 4) % 4) * D + bx * 4 + vi % 4;
-      *reinterpret_cast<uint4 *>(dt + vi * COUT + piece * 8) =
-          *reinterpret_cast<const uint4 *>(dout + v * COUT + piece * 8);
+    const bf16 *ds = dout + (int64_t)s * D * D * D * COUT;
+    for (int p = threadIdx.x; p < G::kVox * (COUT / 8); p += G::kThreads) {
+      const int v = p / (COUT / 8), c = p % (COUT / 8);
+      const int x = x0 + v % BX, y = y0 + (v / BX) % BY, z = z0 + v / (BX * BY);
+      cp_async16(dt + c * G::kDoutPlane + v * 16, ds + (((int64_t)z * D + y) * D + x) * COUT + c * 8);
     }
+  };
+
+  float acc[9][NM][2][4], accb[NM][4];
+#pragma unroll
+  for (int m = 0; m < NM; ++m) {
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) acc[t][m][h][0] = acc[t][m][h][1] = acc[t][m][h][2] = acc[t][m][h][3] = 0.f;
+    accb[m][0] = accb[m][1] = accb[m][2] = accb[m][3] = 0.f;
+  }
+  const bool bias = blockIdx.y == 0 && dz == 0;
+  const int bk = (lane & 7) + ((lane >> 3) & 1) * 8, bhalf = (lane >> 4) & 1;  // B rows: voxel bk, channel half
+  const int ak = (lane & 7) + ((lane >> 4) & 1) * 8, ahalf = (lane >> 3) & 1;  // A rows
+  int buf = 0;
+  if (blockIdx.x < nbricks) stage(blockIdx.x, 0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int bi = blockIdx.x; bi < nbricks; bi += gridDim.x, buf ^= 1) {
+    if (bi + (int)gridDim.x < nbricks) stage(bi + gridDim.x, buf ^ 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
+    const uint32_t halo = smem_u32(smem + buf * G::kStage), dt = halo + 2 * G::kHaloPlane;
+#pragma unroll 1
+    for (int ch = kw; ch < G::kVox / 16; ch += G::KW) {
+      uint32_t a[NM][4];
 #pragma unroll
-    for (int i = 0; i < MAXT; ++i) {
-      const int tile = warp + 8 * i;
-      if (tile < TILES) {
-        const int tl = tile / (NMB * NJP), r = tile % (NMB * NJP), mb = r / NJP, jp = r % NJP;
-        const int t = t0 + tl;
-        const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
+      for (int m = 0; m < NM; ++m)
+        ldsm_x4_t(dt + (2 * (mb0 + m) + ahalf) * G::kDoutPlane + (ch * 16 + ak) * 16, a[m][0], a[m][1], a[m][2],
+                  a[m][3]);
+      const int v = ch * 16 + bk;
+      const uint32_t hb = halo + bhalf * G::kHaloPlane +
+                          ((v / (BX * BY) + dz) * (G::HX * G::HY) + ((v / BX) % BY) * G::HX + v % BX) * 16;
 #pragma unroll
-        for (int k16 = 0; k16 < 4; ++k16) {
-          // A = dout^T (co x voxel) from dt [voxel][co] via ldmatrix.trans
-          const int av = k16 * 16 + (lane & 7) + ((lane >> 4) & 1) * 8;
-          const int aco = mb * 16 + ((lane >> 3) & 1) * 8;
-          uint32_t a0, a1, a2, a3;
-          ldsm_x4_t(smem_u32(dt + av * COUT + aco), a0, a1, a2, a3);
-          // B = in shifted by the tap (voxel x ci) from halo rows via ldmatrix.trans
-          const int bv = k16 * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-          const int hrow = ((bv / 16 + dz + 1) * 6 + ((bv / 4) % 4 + dy + 1)) * 6 + (bv % 4 + dx + 1);
-          const int ci = jp * 16 + ((lane >> 4) & 1) * 8;
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4_t(smem_u32(halo + hrow * CIN + ci), b0, b1, b2, b3);
-          mma16816(acc[i][0], a0, a1, a2, a3, b0, b1);
-          mma16816(acc[i][1], a0, a1, a2, a3, b2, b3);
+      for (int t = 0; t < 9; ++t) {
+        uint32_t b0, b1, b2, b3;
+        ldsm_x4_t(hb + ((t / 3) * G::HX + t % 3) * 16, b0, b1, b2, b3);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+          mma16816(acc[t][m][0], a[m][0], a[m][1], a[m][2], a[m][3], b0, b1);
+          mma16816(acc[t][m][1], a[m][0], a[m][1], a[m][2], a[m][3], b2, b3);
         }
       }
+      if (bias) {
+        constexpr uint32_t kOnes = 0x3F803F80u;  // bf16 1, 1
+#pragma unroll
+        for (int m = 0; m < NM; ++m) mma16816(accb[m], a[m][0], a[m][1], a[m][2], a[m][3], kOnes, kOnes);
+      }
     }
     __syncthreads();
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // the KW partial sums of each (tap, co, ci), then one red.v2 per pair of ci
+  float *red = reinterpret_cast<float *>(smem);  // [27][COUT][16]
   const int g = lane >> 2, q = lane & 3;
+#pragma unroll 1
+  for (int w = 0; w < G::KW; ++w) {
+    if (kw == w) {
 #pragma unroll
-  for (int i = 0; i < MAXT; ++i) {
-    const int tile = warp + 8 * i;
-    if (tile >= TILES) continue;
-    const int tl = tile / (NMB * NJP), r = tile % (NMB * NJP), mb = r / NJP, jp = r % NJP;
-    const int t = t0 + tl;
+      for (int t = 0; t < 9; ++t)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int ci = (2 * jp + h) * 8 + q * 2;
+        for (int m = 0; m < NM; ++m)
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        const int co = mb * 16 + g + hh * 8;
-        float *dst = dW + ((int64_t)co * 27 + t) * CIN + ci;
-        atomicAdd(dst, acc[i][h][2 * hh]);
-        atomicAdd(dst + 1, acc[i][h][2 * hh + 1]);
-      }
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              float2 *r = reinterpret_cast<float2 *>(red + ((dz * 9 + t) * COUT + (mb0 + m) * 16 + g + 8 * hh) * 16 +
+                                                     8 * h + 2 * q);
+              float2 x = make_float2(acc[t][m][h][2 * hh], acc[t][m][h][2 * hh + 1]);
+              if (w > 0) {
+                const float2 o = *r;
+                x.x += o.x;
+                x.y += o.y;
+              }
+              *r = x;
+            }
     }
+    __syncthreads();
   }
+  for (int p = threadIdx.x; p < 27 * COUT * 8; p += G::kThreads) {
+    const int j = p & 7, co = (p >> 3) % COUT, t = p / (8 * COUT);
+    const float2 x = reinterpret_cast<const float2 *>(red)[p];
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dW + ((int64_t)co * 27 + t) * CIN + c_first + 2 * j),
+                 "f"(x.x), "f"(x.y)
+                 : "memory");
+  }
+  if (bias && q == 0)
+#pragma unroll
+    for (int m = 0; m < NM; ++m)
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) atomicAdd(db + (mb0 + m) * 16 + g + 8 * hh, accb[m][2 * hh]);
 }
 
 // ---- per-sample input statistics and the network input
@@ -304,23 +388,25 @@ __global__ void k_pool(const bf16 *__restrict__ in, int D, int C, int B, bf16 *_
   }
 }
 
-// out [B][D^3][Ca+Cb] = [nearest-upsampled a (D/2 grid, Ca), b (D grid, Cb)]
+// out [B][D^3][Ca+Cb] = [nearest-upsampled a (D/2 grid, Ca), b (D grid, Cb)],
+// 8 channels (16 bytes) per thread
 __global__ void k_up_concat(const bf16 *__restrict__ a, int Ca, const bf16 *__restrict__ b, int Cb, int D, int B,
                             bf16 *__restrict__ out) {
-  const int C = Ca + Cb, Dh = D / 2;
-  const int64_t total = (int64_t)B * D * D * D * C;
+  const int C8 = (Ca + Cb) / 8, Ca8 = Ca / 8, Dh = D / 2;
+  const int64_t total = (int64_t)B * D * D * D * C8;
+  const uint4 *av = reinterpret_cast<const uint4 *>(a), *bv = reinterpret_cast<const uint4 *>(b);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % C);
-    const int64_t v = e / C;
-    const int64_t s = v / ((int64_t)D * D * D);
-    const int64_t r = v % ((int64_t)D * D * D);
-    if (c < Ca) {
-      const int z = (int)(r / (D * D)), y = (int)((r / D) % D), x = (int)(r % D);
-      const int64_t u = s * Dh * Dh * Dh + ((int64_t)(z >> 1) * Dh + (y >> 1)) * Dh + (x >> 1);
-      out[e] = a[u * Ca + c];
+    const int64_t v = e / C8;
+    const int c = (int)(e - v * C8);
+    uint4 x;
+    if (c < Ca8) {
+      const int xx = (int)(v % D), y = (int)((v / D) % D);
+      const int64_t sz = v / ((int64_t)D * D);  // sample * D + z, D even
+      x = av[(((sz >> 1) * Dh + (y >> 1)) * Dh + (xx >> 1)) * Ca8 + c];
     } else {
-      out[e] = b[v * Cb + (c - Ca)];
+      x = bv[v * (Cb / 8) + (c - Ca8)];
     }
+    reinterpret_cast<uint4 *>(out)[e] = x;
   }
 }
 
@@ -339,29 +425,42 @@ __global__ void k_head(const bf16 *__restrict__ d0, const float *__restrict__ hw
 }
 
 // loss = mean (delta - target)^2, target = (phi_next - phi_prev) / rms;
-// ddelta = 2 (delta - target) / (B V); dact = bf16(ddelta w); head grads.
-__global__ void k_head_grad(const bf16 *__restrict__ d0, const float *__restrict__ hw, const float *__restrict__ delta,
-                            const float *__restrict__ phi_prev, const float *__restrict__ phi_next,
-                            const float *__restrict__ norm, int64_t V, int B, bf16 *__restrict__ dact,
-                            float *__restrict__ ghw, float *__restrict__ ghb, double *__restrict__ loss) {
-  __shared__ float sh[17][32];
+// ddelta = 2 (delta - target) / (B V); dact = bf16(ddelta w) where d0 > 0,
+// else 0 (the ReLU derivative); head grads.  One voxel (32 bytes of d0 and
+// dact) per thread and step; the 18 block sums are formed by few blocks.
+__global__ void __launch_bounds__(256) k_head_grad(const bf16 *__restrict__ d0, const float *__restrict__ hw,
+                                                  const float *__restrict__ delta, const float *__restrict__ phi_prev,
+                                                  const float *__restrict__ phi_next, const float *__restrict__ norm,
+                                                  int64_t V, int B, bf16 *__restrict__ dact, float *__restrict__ ghw,
+                                                  float *__restrict__ ghb, double *__restrict__ loss) {
+  __shared__ float sh[17][8];
   const int64_t total = (int64_t)B * V;
   const float inv_n = 1.f / (float)total;
-  float acc[17];
+  float acc[17], w[16];
 #pragma unroll
   for (int c = 0; c < 17; ++c) acc[c] = 0.f;
+#pragma unroll
+  for (int c = 0; c < 16; ++c) w[c] = hw[c];
   double l = 0.0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    __align__(16) __nv_bfloat162 d[8], o[8];
+    reinterpret_cast<uint4 *>(d)[0] = __ldg(reinterpret_cast<const uint4 *>(d0 + e * 16));
+    reinterpret_cast<uint4 *>(d)[1] = __ldg(reinterpret_cast<const uint4 *>(d0 + e * 16) + 1);
     const float target = (phi_next[e] - phi_prev[e]) / norm[3 * (e / V) + 2];
     const float diff = delta[e] - target;
     l += (double)diff * diff;
     const float dd = 2.f * diff * inv_n;
     acc[16] += dd;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      acc[c] = fmaf(__bfloat162float(d0[e * 16 + c]), dd, acc[c]);
-      dact[e * 16 + c] = __float2bfloat16_rn(dd * hw[c]);
+    for (int q = 0; q < 8; ++q) {
+      const float x0 = __low2float(d[q]), x1 = __high2float(d[q]);
+      acc[2 * q] = fmaf(x0, dd, acc[2 * q]);
+      acc[2 * q + 1] = fmaf(x1, dd, acc[2 * q + 1]);
+      o[q] = __floats2bfloat162_rn(x0 > 0.f ? dd * w[2 * q] : 0.f, x1 > 0.f ? dd * w[2 * q + 1] : 0.f);
     }
+    uint4 *dst = reinterpret_cast<uint4 *>(dact + e * 16);
+    dst[0] = reinterpret_cast<const uint4 *>(o)[0];
+    dst[1] = reinterpret_cast<const uint4 *>(o)[1];
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -375,59 +474,73 @@ __global__ void k_head_grad(const bf16 *__restrict__ d0, const float *__restrict
   __syncthreads();
   if (threadIdx.x < 17) {
     float v = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[threadIdx.x][w];
+    for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) v += sh[threadIdx.x][w2];
     if (threadIdx.x < 16) atomicAdd(ghw + threadIdx.x, v); else atomicAdd(ghb, v);
   }
 }
 
-// g = bf16(g * (act > 0)) in place (ReLU derivative from the stored output)
-__global__ void k_relu_mask(bf16 *__restrict__ g, const bf16 *__restrict__ act, int64_t n) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    if (!(__bfloat162float(act[e]) > 0.f)) g[e] = __float2bfloat16_rn(0.f);
+// bf16 x 8 with entries zeroed where act is not above 0 (the ReLU derivative)
+__device__ __forceinline__ uint4 pack_masked(const float v[8], const bf16 *act) {
+  __align__(16) __nv_bfloat162 o[4], a[4];
+  *reinterpret_cast<uint4 *>(a) = __ldg(reinterpret_cast<const uint4 *>(act));
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    o[q] = __floats2bfloat162_rn(__low2float(a[q]) > 0.f ? v[2 * q] : 0.f, __high2float(a[q]) > 0.f ? v[2 * q + 1] : 0.f);
+  return *reinterpret_cast<const uint4 *>(o);
 }
-
-// db[c] += sum_v g[v][c]
-__global__ void k_bias_grad(const bf16 *__restrict__ g, int64_t rows, int C, float *__restrict__ db) {
-  const int c = threadIdx.x % C;
-  const int lanes = blockDim.x / C;
-  const int r0 = threadIdx.x / C;
-  float s = 0.f;
-  for (int64_t r = blockIdx.x * (int64_t)lanes + r0; r < rows; r += (int64_t)gridDim.x * lanes)
-    s += __bfloat162float(g[r * C + c]);
-  if (r0 < lanes) atomicAdd(db + c, s);
-}
-
-// gradient split of a concat [up(a) (Ca), b (Cb)] on the D grid:
-//   da[u][c] = bf16(sum over the 8 children of dcat[..][c]), c < Ca  (D/2 grid)
-__global__ void k_up_grad(const bf16 *__restrict__ dcat, int Ca, int Cb, int D, int B, bf16 *__restrict__ da) {
-  const int C = Ca + Cb, Dh = D / 2;
-  const int64_t total = (int64_t)B * Dh * Dh * Dh * Ca;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % Ca);
-    const int64_t u = e / Ca;
-    const int64_t s = u / ((int64_t)Dh * Dh * Dh), r = u % ((int64_t)Dh * Dh * Dh);
-    const int z = (int)(r / (Dh * Dh)), y = (int)((r / Dh) % Dh), x = (int)(r % Dh);
-    float acc = 0.f;
-    for (int k = 0; k < 8; ++k) {
-      const int64_t v = s * D * D * D + ((int64_t)(2 * z + (k >> 2)) * D + 2 * y + ((k >> 1) & 1)) * D + 2 * x + (k & 1);
-      acc += __bfloat162float(dcat[v * C + c]);
-    }
-    da[e] = __float2bfloat16_rn(acc);
+__device__ __forceinline__ void unpack8(const bf16 *p, float v[8]) {
+  __align__(16) __nv_bfloat162 a[4];
+  *reinterpret_cast<uint4 *>(a) = __ldg(reinterpret_cast<const uint4 *>(p));
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    v[2 * q] = __low2float(a[q]);
+    v[2 * q + 1] = __high2float(a[q]);
   }
 }
 
-// skip gradient: ds[v][c] = bf16(dcat[v][Ca + c] + dpool[parent(v)][c] / 8)
-__global__ void k_skip_grad(const bf16 *__restrict__ dcat, int Ca, int Cb, const bf16 *__restrict__ dpool, int D,
-                            int B, bf16 *__restrict__ ds) {
-  const int C = Ca + Cb, Dh = D / 2;
-  const int64_t total = (int64_t)B * D * D * D * Cb;
+// gradient split of a concat [up(a) (Ca), b (Cb)] on the D grid, 8 channels
+// (16 bytes) per thread:
+//   da[u][c] = bf16(sum over the 8 children of dcat[..][c]), c < Ca (D/2
+//   grid), 0 where the activation a is
+__global__ void k_up_grad(const bf16 *__restrict__ dcat, int Ca, int Cb, const bf16 *__restrict__ act, int D, int B,
+                          bf16 *__restrict__ da) {
+  const int C = Ca + Cb, Ca8 = Ca / 8, Dh = D / 2;
+  const int64_t total = (int64_t)B * Dh * Dh * Dh * Ca8;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % Cb);
-    const int64_t v = e / Cb;
-    const int64_t s = v / ((int64_t)D * D * D), r = v % ((int64_t)D * D * D);
-    const int z = (int)(r / (D * D)), y = (int)((r / D) % D), x = (int)(r % D);
-    const int64_t u = s * Dh * Dh * Dh + ((int64_t)(z >> 1) * Dh + (y >> 1)) * Dh + (x >> 1);
-    ds[e] = __float2bfloat16_rn(__bfloat162float(dcat[v * C + Ca + c]) + __bfloat162float(dpool[u * Cb + c]) * 0.125f);
+    const int64_t u = e / Ca8;
+    const int c = (int)(e - u * Ca8) * 8;
+    const int x = (int)(u % Dh), y = (int)((u / Dh) % Dh);
+    const int64_t sz = u / ((int64_t)Dh * Dh);  // sample * Dh + z
+    const bf16 *p = dcat + ((2 * sz * D + 2 * y) * D + 2 * x) * C + c;
+    float acc[8] = {};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      float v[8];
+      unpack8(p + (((int64_t)(k >> 2) * D + ((k >> 1) & 1)) * D + (k & 1)) * C, v);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[q] += v[q];
+    }
+    *reinterpret_cast<uint4 *>(da + e * 8) = pack_masked(acc, act + e * 8);
+  }
+}
+
+// skip gradient: ds[v][c] = bf16(dcat[v][Ca + c] + dpool[parent(v)][c] / 8),
+// 0 where the skip's activation is; 8 channels per thread
+__global__ void k_skip_grad(const bf16 *__restrict__ dcat, int Ca, int Cb, const bf16 *__restrict__ dpool,
+                            const bf16 *__restrict__ act, int D, int B, bf16 *__restrict__ ds) {
+  const int C = Ca + Cb, Cb8 = Cb / 8, Dh = D / 2;
+  const int64_t total = (int64_t)B * D * D * D * Cb8;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = e / Cb8;
+    const int c = (int)(e - v * Cb8) * 8;
+    const int x = (int)(v % D), y = (int)((v / D) % D);
+    const int64_t sz = v / ((int64_t)D * D);  // sample * D + z, D even
+    float a[8], b[8];
+    unpack8(dcat + v * C + Ca + c, a);
+    unpack8(dpool + (((sz >> 1) * Dh + (y >> 1)) * Dh + (x >> 1)) * Cb + c, b);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = a[q] + b[q] * 0.125f;
+    *reinterpret_cast<uint4 *>(ds + e * 8) = pack_masked(a, act + e * 8);
   }
 }
 
@@ -482,16 +595,25 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
   }
 }
 
-// bf16 weight copies: W [co][t][ci] and WT [ci][t][co] from the master slice
-__global__ void k_cast_w(const float *__restrict__ w, int co_n, int ci_n, bf16 *__restrict__ W, bf16 *__restrict__ WT) {
-  const int64_t n = (int64_t)co_n * 27 * ci_n;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int ci = (int)(e % ci_n);
-    const int t = (int)((e / ci_n) % 27);
-    const int co = (int)(e / (27 * ci_n));
-    const bf16 x = __float2bfloat16_rn(w[e]);
-    W[e] = x;
-    WT[((int64_t)ci * 27 + t) * co_n + co] = x;
+// bf16 weight copies of every layer (blockIdx.y) from the master vector: W
+// [co][t][ci], WT [ci][t][co], and both arranged for the tcgen05 kernels.
+struct WeightPlan {
+  struct Layer {
+    const float *w;
+    int co, ci;
+    bf16 *W, *WT, *WI, *WTI;
+  } l[10];
+};
+__global__ void k_prepare_weights(const __grid_constant__ WeightPlan P) {
+  const WeightPlan::Layer &L = P.l[blockIdx.y];
+  const int n = L.co * 27 * L.ci;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int ci = e % L.ci, t = (e / L.ci) % 27, co = e / (27 * L.ci);
+    const bf16 x = __float2bfloat16_rn(L.w[e]);
+    L.W[e] = x;
+    L.WT[(ci * 27 + t) * L.co + co] = x;
+    L.WI[tc::image_index(L.co, 1, co, t, ci)] = x;
+    L.WTI[tc::image_index(L.ci, -1, ci, t, co)] = x;
   }
 }
 
@@ -591,7 +713,8 @@ void conv_tc_launch(cmg_unet *U, const bf16 *in, int K, const bf16 *skip, int Cb
 }
 
 template <int NT, int SIGN, bool BR>
-void conv_launch(cmg_unet *U, const bf16 *in, int K, const bf16 *W, const float *bias, bf16 *out, int D, int B) {
+void conv_launch(cmg_unet *U, const bf16 *in, int K, const bf16 *W, const float *bias, const bf16 *mask, bf16 *out,
+                 int D, int B) {
   const size_t smem = (216 * 16 + (size_t)NT * 8 * 27 * 16) * sizeof(bf16);
   static bool attr = false;
   if (!attr) {
@@ -600,7 +723,7 @@ void conv_launch(cmg_unet *U, const bf16 *in, int K, const bf16 *W, const float 
   }
   const int nb = (D / 4) * (D / 4) * (D / 4);
   LaunchScope ls(U->ctx, SIGN > 0 ? K_CONV_FWD : K_CONV_DGRAD, 0.0, 2.0 * 27 * K * NT * 8 * (double)D * D * D * B);
-  k_conv<NT, SIGN, BR><<<dim3(nb, B), kConvThreads, smem, U->ctx->stream>>>(in, K, W, bias, out, D);
+  k_conv<NT, SIGN, BR><<<dim3(nb, B), kConvThreads, smem, U->ctx->stream>>>(in, K, W, bias, mask, out, D);
   CMG_CUDA(cudaGetLastError());
 }
 
@@ -643,17 +766,21 @@ bool conv_tc(cmg_unet *U, const bf16 *in, int K, const bf16 *skip, int Cb, const
 }
 
 // Convolution of layer l: forward (in = activations, N = cout) or input
-// gradient (in = output gradient, N = cin).
-void conv(cmg_unet *U, int l, const bf16 *in, int K, const float *bias, bf16 *out, int N, int D, int B, bool fwd) {
+// gradient (in = output gradient, N = cin; mask: the activations whose ReLU
+// derivative multiplies it, or nullptr).
+void conv(cmg_unet *U, int l, const bf16 *in, int K, const float *bias, const bf16 *mask, bf16 *out, int N, int D,
+          int B, bool fwd) {
   if (tc_eligible(U, N, D)) {
-    conv_tc(U, in, K, nullptr, 0, fwd ? U->WI[l] : U->WTI[l], bias, out, N, D, B, fwd);
+    tc::ConvEpi ep;
+    ep.mask = mask;
+    conv_tc(U, in, K, nullptr, 0, fwd ? U->WI[l] : U->WTI[l], bias, out, N, D, B, fwd, ep);
     return;
   }
   const bf16 *W = fwd ? U->W[l] : U->WT[l];
 #define CMG_CONV(NT)                                                             \
   case NT:                                                                       \
-    if (fwd) conv_launch<NT, 1, true>(U, in, K, W, bias, out, D, B);             \
-    else conv_launch<NT, -1, false>(U, in, K, W, nullptr, out, D, B);            \
+    if (fwd) conv_launch<NT, 1, true>(U, in, K, W, bias, nullptr, out, D, B);    \
+    else conv_launch<NT, -1, false>(U, in, K, W, nullptr, mask, out, D, B);      \
     break;
   switch (N / 8) {
     CMG_CONV(2)
@@ -666,40 +793,37 @@ void conv(cmg_unet *U, int l, const bf16 *in, int K, const float *bias, bf16 *ou
 #undef CMG_CONV
 }
 
-template <int CIN, int COUT, int TG>
-void wgrad_launch(cmg_unet *U, const bf16 *dout, const bf16 *in, float *dW, int D, int B) {
-  const size_t smem = ((size_t)216 * CIN + 64 * (size_t)COUT) * sizeof(bf16);
+template <int COUT, int BX, int BY, int BZ>
+void wgrad_launch(cmg_unet *U, const bf16 *dout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW, float *db,
+                  int D, int B) {
+  using G = WgradGeom<COUT, BX, BY, BZ>;
   static int attr_dev = -1;
   if (attr_dev != U->ctx->device) {
-    CMG_CUDA(cudaFuncSetAttribute(k_conv_wgrad<CIN, COUT, TG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+    CMG_CUDA(cudaFuncSetAttribute(k_conv_wgrad<COUT, BX, BY, BZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  G::kSmem));
     attr_dev = U->ctx->device;
   }
-  const int nbricks = B * (D / 4) * (D / 4) * (D / 4);
-  const int gy = 27 / TG;
-  const int bx = std::max(1, std::min(nbricks, 4 * U->ctx->num_sms / gy));
-  const int per_block = (nbricks + bx - 1) / bx;
-  const int blocks = (nbricks + per_block - 1) / per_block;
-  LaunchScope ls(U->ctx, K_CONV_WGRAD, 0.0, 2.0 * 27 * COUT * CIN * (double)D * D * D * B);
-  k_conv_wgrad<CIN, COUT, TG><<<dim3(blocks, gy), kWgThreads, smem, U->ctx->stream>>>(dout, in, dW, D, nbricks,
-                                                                                     per_block);
+  const int nbricks = B * (D / BX) * (D / BY) * (D / BZ), slices = Cin / 16;
+  const int blocks = std::max(1, std::min(nbricks, U->ctx->num_sms / slices));
+  LaunchScope ls(U->ctx, K_CONV_WGRAD, 0.0, 2.0 * 27 * COUT * Cin * (double)D * D * D * B);
+  k_conv_wgrad<COUT, BX, BY, BZ><<<dim3(blocks, slices), G::kThreads, G::kSmem, U->ctx->stream>>>(
+      dout, in, Cin, skip, Cb, dW, db, D, nbricks);
   CMG_CUDA(cudaGetLastError());
 }
 
-// Taps per block: as many (27, 9 or 3) as keep the accumulators of a warp
-// within 12 tiles (96 registers).
-void wgrad(cmg_unet *U, const bf16 *dout, int Cout, const bf16 *in, int Cin, float *dW, int D, int B) {
-#define CMG_WG(CI, CO, TG)                                      \
-  if (Cin == CI && Cout == CO) {                                \
-    wgrad_launch<CI, CO, TG>(U, dout, in, dW, D, B);            \
-    return;                                                     \
+// Weight and bias gradients; bricks of 8 x 8 x 4 voxels, 4 x 4 x 4 on grids
+// that 8 does not divide.  skip: see k_conv_wgrad.
+void wgrad(cmg_unet *U, const bf16 *dout, int Cout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW,
+           float *db, int D, int B) {
+#define CMG_WG(CO)                                                                        \
+  if (Cout == CO) {                                                                       \
+    if (D % 8 == 0) wgrad_launch<CO, 8, 8, 4>(U, dout, in, Cin, skip, Cb, dW, db, D, B);  \
+    else wgrad_launch<CO, 4, 4, 4>(U, dout, in, Cin, skip, Cb, dW, db, D, B);             \
+    return;                                                                               \
   }
-  CMG_WG(16, 16, 27)
-  CMG_WG(16, 32, 27)
-  CMG_WG(32, 32, 9)
-  CMG_WG(32, 64, 9)
-  CMG_WG(64, 64, 3)
-  CMG_WG(96, 32, 3)
-  CMG_WG(48, 16, 27)
+  CMG_WG(16)
+  CMG_WG(32)
+  CMG_WG(64)
 #undef CMG_WG
   throw Error(CMG_ERR_INVALID_ARG, "unsupported channel count");
 }
@@ -724,13 +848,10 @@ int64_t vox(const cmg_unet *U, int lvl) {
 void prepare_weights(cmg_unet *U) {
   if (U->weights_ready) return;
   cudaStream_t s = U->ctx->stream;
-  for (int l = 0; l < 10; ++l) {
-    const LayerSpec &L = kLayers[l];
-    const int64_t n = (int64_t)L.cout * 27 * L.cin;
-    k_cast_w<<<gsz(n), 256, 0, s>>>(U->params + layer_offset(l), L.cout, L.cin, U->W[l], U->WT[l]);
-    tc::k_weight_image<<<gsz(n), 256, 0, s>>>(U->W[l], L.cout, L.cin, 1, U->WI[l]);
-    tc::k_weight_image<<<gsz(n), 256, 0, s>>>(U->WT[l], L.cin, L.cout, -1, U->WTI[l]);
-  }
+  WeightPlan P;
+  for (int l = 0; l < 10; ++l)
+    P.l[l] = {U->params + layer_offset(l), kLayers[l].cout, kLayers[l].cin, U->W[l], U->WT[l], U->WI[l], U->WTI[l]};
+  k_prepare_weights<<<dim3(32, 10), 256, 0, s>>>(P);
   CMG_CUDA(cudaGetLastError());
   U->weights_ready = true;
 }
@@ -739,21 +860,29 @@ const float *bias_of(cmg_unet *U, int l) {
   return U->params + layer_offset(l) + (int64_t)kLayers[l].cout * 27 * kLayers[l].cin;
 }
 
-// Forward pass on U->in_rho / U->in_phi (B samples); leaves activations,
+// Device arrays of one call: inputs (base may be the field, next only in
+// training) and outputs (pred, delta or nullptr).  Device-memory arguments are
+// read and written in place, host-memory ones through the network's buffers.
+struct Fields {
+  const float *rho, *phi, *base, *next;
+  float *pred, *delta;
+};
+
+// Forward pass on F.rho / F.phi (B samples); leaves activations,
 // delta and (if phi_pred) phi_prev + rms * delta.
-void forward(cmg_unet *U, int B, float *phi_pred, bool training) {
+void forward(cmg_unet *U, int B, const Fields &F, bool training) {
   cudaStream_t s = U->ctx->stream;
   prepare_weights(U);
   const int64_t V0 = vox(U, 0);
   CMG_CUDA(cudaMemsetAsync(U->stats, 0, sizeof(double) * 3 * B, s));
-  k_stats<<<dim3(64, B), 256, 0, s>>>(U->in_rho, U->in_phi, V0, U->stats);
+  k_stats<<<dim3(64, B), 256, 0, s>>>(F.rho, F.phi, V0, U->stats);
   k_norm<<<1, (B + 31) / 32 * 32, 0, s>>>(U->stats, V0, B, U->out_scale, U->norm, U->norm + 3 * U->max_batch);
-  k_input<<<dim3(gsz(V0), B), 256, 0, s>>>(U->in_rho, U->in_phi, V0, U->norm, U->norm + 3 * U->max_batch, U->x);
+  k_input<<<dim3(gsz(V0), B), 256, 0, s>>>(F.rho, F.phi, V0, U->norm, U->norm + 3 * U->max_batch, U->x);
   CMG_CUDA(cudaGetLastError());
-  const int D0 = dim_of(U, 0), D1 = dim_of(U, 1), D2 = dim_of(U, 2);
+  const int D0 = dim_of(U, 0), D1 = dim_of(U, 1);
   auto layer = [&](int l, const bf16 *in, bf16 *out) {
     const LayerSpec &L = kLayers[l];
-    conv(U, l, in, L.cin, bias_of(U, l), out, L.cout, dim_of(U, L.lvl), B, true);
+    conv(U, l, in, L.cin, bias_of(U, l), nullptr, out, L.cout, dim_of(U, L.lvl), B, true);
   };
   // encoder convolution + 2x2x2 pooling (fused into the tcgen05 epilogue
   // where the bricks allow it)
@@ -776,13 +905,13 @@ void forward(cmg_unet *U, int B, float *phi_pred, bool training) {
   layer_pool(3, U->a[2], U->a[3], U->p1);  // s1
   layer(4, U->p1, U->a[4]);
   layer(5, U->a[4], U->a[5]);
-  // decoder convolutions: in inference the tcgen05 kernels read the
-  // upsampled coarse map and the skip map directly; training keeps the
-  // concatenation (the backward pass needs it)
+  // decoder convolutions: the tcgen05 kernels read the upsampled coarse map
+  // and the skip map directly (so does the weight gradient); the warp-level
+  // kernels read the concatenation
   auto up_layer = [&](int l, const bf16 *coarse, int Ca, const bf16 *skipm, int Cb, bf16 *cat, bf16 *out) {
     const LayerSpec &L = kLayers[l];
     const int D = dim_of(U, L.lvl);
-    if (!training && tc_eligible(U, L.cout, D)) {
+    if (tc_eligible(U, L.cout, D)) {
       conv_tc(U, coarse, Ca + Cb, skipm, Cb, U->WI[l], bias_of(U, l), out, L.cout, D, B, true);
       return;
     }
@@ -797,70 +926,75 @@ void forward(cmg_unet *U, int B, float *phi_pred, bool training) {
     // last convolution + head in one kernel; its activations are not kept
     tc::ConvEpi ep;
     ep.hw = hw;
-    ep.base = U->in_base;
+    ep.base = F.base;
     ep.norm = U->norm;
-    ep.delta = U->delta;
-    ep.pred = phi_pred;
+    ep.delta = F.delta;
+    ep.pred = F.pred;
     ep.store_out = 0;
     conv_tc(U, U->a[8], 16, nullptr, 0, U->WI[9], bias_of(U, 9), U->a[9], 16, D0, B, true, ep);
   } else {
     layer(9, U->a[8], U->a[9]);
-    k_head<<<gsz(B * V0), 256, 0, s>>>(U->a[9], hw, hw + 16, U->in_base, U->norm, V0, B, U->delta, phi_pred);
+    k_head<<<gsz(B * V0), 256, 0, s>>>(U->a[9], hw, hw + 16, F.base, U->norm, V0, B, F.delta, F.pred);
   }
   CMG_CUDA(cudaGetLastError());
-  (void)D2;
 }
 
 // Backward pass after forward(): gradients (summed over the batch's voxels,
 // loss = mean over all voxels) into U->grads; loss into U->loss.
-void backward(cmg_unet *U, int B) {
+void backward(cmg_unet *U, int B, const Fields &F) {
   cudaStream_t s = U->ctx->stream;
   const int64_t V0 = vox(U, 0), V1 = vox(U, 1), V2 = vox(U, 2);
-  const int D0 = dim_of(U, 0), D1 = dim_of(U, 1), D2 = dim_of(U, 2);
+  const int D0 = dim_of(U, 0), D1 = dim_of(U, 1);
   CMG_CUDA(cudaMemsetAsync(U->grads, 0, sizeof(float) * U->np, s));
   CMG_CUDA(cudaMemsetAsync(U->loss, 0, sizeof(double), s));
   float *ghw = U->grads + layer_offset(10);
-  k_head_grad<<<gsz(B * V0), 256, 0, s>>>(U->a[9], U->params + layer_offset(10), U->delta, U->in_base, U->in_next,
-                                          U->norm, V0, B, U->g0, ghw, ghw + 16, U->loss);
+  k_head_grad<<<std::min<int64_t>(gsz(B * V0), 4 * U->ctx->num_sms), 256, 0, s>>>(
+      U->a[9], U->params + layer_offset(10), F.delta, F.base, F.next, U->norm, V0, B, U->g0, ghw, ghw + 16,
+      U->loss);
   CMG_CUDA(cudaGetLastError());
-  // back through layer l: g (grad of its output, bf16) -> grad of its input
-  auto back = [&](int l, bf16 *g, const bf16 *in, bf16 *gin) {
+  // back through layer l: g (gradient of its pre-activation, bf16) -> its
+  // weights' and biases' gradients and the gradient gin of its input, times
+  // the ReLU derivative of the layer that made the input (below) if that
+  // layer alone did
+  auto back = [&](int l, const bf16 *g, const bf16 *in, const bf16 *skip, int Cb, bf16 *gin, const bf16 *below) {
     const LayerSpec &L = kLayers[l];
     const int D = dim_of(U, L.lvl);
-    const int64_t rows = (int64_t)B * vox(U, L.lvl);
-    k_relu_mask<<<gsz(rows * L.cout), 256, 0, s>>>(g, U->a[l], rows * L.cout);
     float *gw = U->grads + layer_offset(l);
-    k_bias_grad<<<256, 256, 0, s>>>(g, rows, L.cout, gw + (int64_t)L.cout * 27 * L.cin);
-    CMG_CUDA(cudaGetLastError());
-    wgrad(U, g, L.cout, in, L.cin, gw, D, B);
-    if (gin) conv(U, l, g, L.cout, nullptr, gin, L.cin, D, B, false);
+    wgrad(U, g, L.cout, in, L.cin, skip, Cb, gw, gw + (int64_t)L.cout * 27 * L.cin, D, B);
+    if (gin) conv(U, l, g, L.cout, nullptr, below, gin, L.cin, D, B, false);
   };
   // decoder level 0
-  back(9, U->g0, U->a[8], U->g1);            // g1 = grad a8 (16 ch, V0)
-  back(8, U->g1, U->c0, U->gc);              // gc = grad c0 (48 ch, V0)
-  k_up_grad<<<gsz(B * V1 * 32), 256, 0, s>>>(U->gc, 32, 16, D0, B, U->gu);  // grad a7 (32 ch, V1)
+  back(9, U->g0, U->a[8], nullptr, 0, U->g1, U->a[8]);           // g1 = grad a8 (16 ch, V0)
+  back(8, U->g1, U->a[7], U->a[1], 16, U->gc, nullptr);          // gc = grad [up a7, a1] (48 ch, V0)
+  k_up_grad<<<gsz(B * V1 * 4), 256, 0, s>>>(U->gc, 32, 16, U->a[7], D0, B, U->gu);  // grad a7 (32 ch, V1)
   // decoder level 1
-  back(7, U->gu, U->a[6], U->gx);            // gx = grad a6 (32 ch, V1)
-  back(6, U->gx, U->c1, U->g0);              // g0 reused: grad c1 (96 ch, V1)
-  k_up_grad<<<gsz(B * V2 * 64), 256, 0, s>>>(U->g0, 64, 32, D1, B, U->gu);  // grad a5 (64 ch, V2)
+  back(7, U->gu, U->a[6], nullptr, 0, U->gx, U->a[6]);           // gx = grad a6 (32 ch, V1)
+  back(6, U->gx, U->a[5], U->a[3], 32, U->g0, nullptr);          // g0 reused: grad [up a5, a3] (96 ch, V1)
+  k_up_grad<<<gsz(B * V2 * 8), 256, 0, s>>>(U->g0, 64, 32, U->a[5], D1, B, U->gu);  // grad a5 (64 ch, V2)
   // bottleneck
-  back(5, U->gu, U->a[4], U->gx);            // grad a4 (64, V2)
-  back(4, U->gx, U->p1, U->gp);              // grad p1 (32, V2)
-  k_skip_grad<<<gsz(B * V1 * 32), 256, 0, s>>>(U->g0, 64, 32, U->gp, D1, B, U->gs1);  // grad s1 = a3
+  back(5, U->gu, U->a[4], nullptr, 0, U->gx, U->a[4]);           // grad a4 (64, V2)
+  back(4, U->gx, U->p1, nullptr, 0, U->gp, nullptr);             // grad p1 (32, V2)
+  k_skip_grad<<<gsz(B * V1 * 4), 256, 0, s>>>(U->g0, 64, 32, U->gp, U->a[3], D1, B, U->gs1);  // grad s1 = a3
   // encoder level 1
-  back(3, U->gs1, U->a[2], U->gx);           // grad a2 (32, V1)
-  back(2, U->gx, U->p0, U->gp);              // grad p0 (16, V1)
-  k_skip_grad<<<gsz(B * V0 * 16), 256, 0, s>>>(U->gc, 32, 16, U->gp, D0, B, U->gs0);  // grad s0 = a1
+  back(3, U->gs1, U->a[2], nullptr, 0, U->gx, U->a[2]);          // grad a2 (32, V1)
+  back(2, U->gx, U->p0, nullptr, 0, U->gp, nullptr);             // grad p0 (16, V1)
+  k_skip_grad<<<gsz(B * V0 * 2), 256, 0, s>>>(U->gc, 32, 16, U->gp, U->a[1], D0, B, U->gs0);  // grad s0 = a1
   // encoder level 0
-  back(1, U->gs0, U->a[0], U->g1);           // grad a0 (16, V0)
-  back(0, U->g1, U->x, nullptr);
+  back(1, U->gs0, U->a[0], nullptr, 0, U->g1, U->a[0]);          // grad a0 (16, V0)
+  back(0, U->g1, U->x, nullptr, 0, nullptr, nullptr);
   CMG_CUDA(cudaGetLastError());
-  (void)D2;
 }
 
 void copy_in(cmg_unet *U, float *dst, const float *src, int64_t n, int mem) {
   CMG_CUDA(cudaMemcpyAsync(dst, src, sizeof(float) * n,
                            mem == CMG_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, U->ctx->stream));
+}
+
+// An input field on the device: src itself, or buf with a copy of host memory.
+const float *field_in(cmg_unet *U, float *buf, const float *src, int64_t n, int mem) {
+  if (mem != CMG_MEM_HOST) return src;
+  copy_in(U, buf, src, n, mem);
+  return buf;
 }
 
 }  // namespace
@@ -1019,14 +1153,17 @@ int cmg_unet_forward(cmg_unet *U, const float *rho, const float *field, const fl
     cudaSetDevice(U->ctx->device);
     const int64_t n = (int64_t)batch * U->D * U->D * U->D;
     cudaStream_t s = U->ctx->stream;
-    cmg::copy_in(U, U->in_rho, rho, n, mem);
-    cmg::copy_in(U, U->in_phi, field, n, mem);
-    cmg::copy_in(U, U->in_base, base ? base : field, n, mem);
-    cmg::forward(U, batch, U->out_phi, false);
-    const cudaMemcpyKind k = mem == CMG_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    if (phi_pred) CMG_CUDA(cudaMemcpyAsync(phi_pred, U->out_phi, sizeof(float) * n, k, s));
-    if (delta) CMG_CUDA(cudaMemcpyAsync(delta, U->delta, sizeof(float) * n, k, s));
-    if (mem == CMG_MEM_HOST) {
+    const bool host = mem == CMG_MEM_HOST;
+    cmg::Fields F = {};
+    F.rho = cmg::field_in(U, U->in_rho, rho, n, mem);
+    F.phi = cmg::field_in(U, U->in_phi, field, n, mem);
+    F.base = base ? cmg::field_in(U, U->in_base, base, n, mem) : F.phi;
+    F.pred = !phi_pred ? nullptr : host ? U->out_phi : phi_pred;
+    F.delta = !delta ? nullptr : host ? U->delta : delta;
+    cmg::forward(U, batch, F, false);
+    if (host) {
+      if (phi_pred) CMG_CUDA(cudaMemcpyAsync(phi_pred, U->out_phi, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
+      if (delta) CMG_CUDA(cudaMemcpyAsync(delta, U->delta, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
       CMG_CUDA(cudaStreamSynchronize(s));
       cmg::check_status(U);
     }
@@ -1041,12 +1178,14 @@ int cmg_unet_gradients(cmg_unet *U, const float *rho, const float *field, const 
     cudaSetDevice(U->ctx->device);
     const int64_t n = (int64_t)batch * U->D * U->D * U->D;
     cudaStream_t s = U->ctx->stream;
-    cmg::copy_in(U, U->in_rho, rho, n, mem);
-    cmg::copy_in(U, U->in_phi, field, n, mem);
-    cmg::copy_in(U, U->in_base, base ? base : field, n, mem);
-    cmg::copy_in(U, U->in_next, target, n, mem);
-    cmg::forward(U, batch, nullptr, true);
-    cmg::backward(U, batch);
+    cmg::Fields F = {};
+    F.rho = cmg::field_in(U, U->in_rho, rho, n, mem);
+    F.phi = cmg::field_in(U, U->in_phi, field, n, mem);
+    F.base = base ? cmg::field_in(U, U->in_base, base, n, mem) : F.phi;
+    F.next = cmg::field_in(U, U->in_next, target, n, mem);
+    F.delta = U->delta;
+    cmg::forward(U, batch, F, true);
+    cmg::backward(U, batch, F);
     const cudaMemcpyKind k = mem == CMG_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     if (grads) CMG_CUDA(cudaMemcpyAsync(grads, U->grads, sizeof(float) * U->np, k, s));
     if (loss) {
