@@ -10,8 +10,14 @@
 // its own add returned.  The add has release and the polling load acquire
 // semantics at GPU scope; the block barriers around them extend the ordering
 // to the CTA's other threads.  A wait longer than budget SM clock cycles
-// records CMG_ERR_TIMEOUT in *err and gives up; once *err holds it, no
-// barrier waits any more, so a failed launch always ends.
+// records CMG_ERR_TIMEOUT in *err and gives up; once *err holds it, a wait
+// that is not over yet ends at its next poll, so a failed launch always ends.
+//
+// A barrier is a chain of L2 round trips (about 0.3 us each): the release of
+// the CTA's stores, the add, the last poll.  The error word is therefore read
+// beside each poll, in flight with it, and not once more after the last one:
+// with that extra read and the two loads of a poll in sequence a barrier of
+// 152 CTAs took 1.26 us.
 #pragma once
 
 #include "cmg.h"
@@ -31,7 +37,13 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
   return v;
 }
 
-// Returns false when this barrier (or an earlier one) gave up.
+__device__ __forceinline__ int ld_relaxed_gpu(const int *p) {
+  int v;
+  asm volatile("ld.relaxed.gpu.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Returns false when this CTA's wait gave up or ended on the error word.
 __device__ __forceinline__ bool grid_barrier(unsigned *word, int *err, long long budget) {
   __shared__ int ok;
   __syncthreads();
@@ -39,10 +51,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned *word, int *err, long long
     ok = 1;
     const unsigned inc = blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1) : 1u;
     const unsigned old = atom_add_release_gpu(word, inc);
-    volatile int *e = err;
     const long long t0 = clock64();
-    while (((ld_acquire_gpu(word) ^ old) & 0x80000000u) == 0u) {
-      if (*e == CMG_ERR_TIMEOUT) {
+    for (;;) {
+      const int e = ld_relaxed_gpu(err);
+      if (((ld_acquire_gpu(word) ^ old) & 0x80000000u) != 0u) break;
+      if (e == CMG_ERR_TIMEOUT) {
         ok = 0;
         break;
       }
@@ -52,7 +65,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned *word, int *err, long long
         break;
       }
     }
-    if (*e == CMG_ERR_TIMEOUT) ok = 0;
   }
   __syncthreads();
   return ok != 0;
