@@ -64,28 +64,44 @@ __device__ __forceinline__ void store4(float *p, const float v[4]) {
 // than five sequential FP64 additions, and does not depend on the order of
 // the operands.  Zero and subnormal operands contribute nothing (a subnormal
 // is below 2^-1022, far under the scale).  The rounding is written out in
-// integer operations: one biased truncation (CMG_FXNORM = 2, the default) or
-// the dropped part compared with half (0); or it is the int64 -> FP64
-// conversion (1).  The alignment below costs ~15 integer instructions per
-// operand; an earlier form (significand assembled with its leading bit,
-// shifted left 7 and right by E - e, negated as (m ^ s) - s) gave the same
-// bits on 10^6 probe sums and ran 15 % slower on GB300.
-// Measured on GB300 (512^3 FP64 colour pass): CMG_FXNORM = 2 0.407 ms
-// against 0.422 ms for 0 (same bits); 1 was slower in the 4 + 2 split
-// (0.486 -> 0.603 ms): the conversion issues on the FP64 pipe.
-#ifndef CMG_FXNORM
-#define CMG_FXNORM 2
-#endif
-// CMG_FXALIGN: 1 = the alignment below; 0 = the earlier form (same bits
-// whenever some operand is 2^-960 or larger).
-#ifndef CMG_FXALIGN
-#define CMG_FXALIGN 1
-#endif
+// integer operations too: the int64 -> FP64 conversion issues on the FP64
+// pipe.  The alignment costs ~15 integer instructions per operand.
 // x >> s with PTX semantics: a shift of 64 or more gives 0.
 __device__ __forceinline__ unsigned long long shr_clamped(unsigned long long x, unsigned s) {
   unsigned long long r;
   asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));
   return r;
+}
+
+// S 2^(E - 1082) rounded to the nearest FP64 value, ties to even; Ex = E << 20
+// with 64 <= E < 0x7FC, |S| < 2^63.
+__device__ __forceinline__ double fixed_round(long long S, int Ex) {
+  const int sg = (int)(S >> 63);  // 0 or -1
+  // |S|, or |S| - 1 for a negative S: the 1 is added with the rounding bias
+  // below.  Where it would change the leading bit or the last kept bit, the
+  // bits rounded off are all zero and the same value comes out.
+  const uint32_t alo = (uint32_t)S ^ (uint32_t)sg, ahi = (uint32_t)((unsigned long long)S >> 32) ^ (uint32_t)sg;
+  if (ahi >= (1u << 21)) {  // leading bit at p = 63 - c > 52: r = p - 52 bits are rounded off
+    const int c = __clz((int)ahi), r = 11 - c;
+    // round half to even by one biased truncation: adding 2^(r-1) - 1 plus
+    // the last kept bit carries into the kept bits exactly when the dropped
+    // part is above half, or equal to it with the kept part odd
+    const uint32_t bias = ((1u << (r - 1)) - 1u) + (__funnelshift_r(alo, ahi, r) & 1u) - (uint32_t)sg;
+    const unsigned long long b = (((unsigned long long)ahi << 32) | alo) + bias;
+    const uint32_t bhi = (uint32_t)(b >> 32);
+    // the kept part carries its leading bit at 2^52 (2^53 after a rounding
+    // carry), which adds the last 1 (or 2) to the exponent field E + p - 59
+    const uint32_t hi = (bhi >> r) + (uint32_t)(Ex + ((3 - c) << 20));
+    return __hiloint2double((int)(hi | ((uint32_t)sg & 0x80000000u)), (int)__funnelshift_r((uint32_t)b, bhi, r));
+  }
+  if (S == 0) return 0.0;
+  const unsigned long long a = S < 0 ? 0ull - (unsigned long long)S : (unsigned long long)S;
+  const int p = 63 - __clzll((long long)a), eb = (Ex >> 20) + p - 59;
+  if (eb <= 0) return ldexp((double)S, (Ex >> 20) - 1082);  // subnormal sum (never in practice)
+  if (p > 52)  // |S| = 2^53 alone, above the test on |S| - 1
+    return __longlong_as_double((long long)(((unsigned long long)eb << 52) + ((S < 0 ? 1ull : 0ull) << 63)));
+  return __longlong_as_double(
+      (long long)(((unsigned long long)(eb - 1) << 52) + (a << (52 - p)) + ((S < 0 ? 1ull : 0ull) << 63)));
 }
 
 template <int N>
@@ -127,17 +143,6 @@ __device__ __forceinline__ double fixed_sum(const double *v) {
   // Negative operands enter as ones' complements; the count of them, added
   // once, completes the two's complements.
   long long S = 0;
-#if CMG_FXALIGN == 0
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const int ek = max(e[k], 1);
-    const uint32_t lead = (hi[k] & 0x7FF00000u) ? 0x100000u : 0u;
-    unsigned long long m = ((unsigned long long)((hi[k] & 0xFFFFFu) | lead) << 32) | lo[k];
-    m = (m << 7) >> min(E - ek, 63);
-    const long long sg = (long long)((int)hi[k] >> 31);
-    S += ((long long)m ^ sg) - sg;
-  }
-#else
   int negs = 0;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
@@ -149,90 +154,28 @@ __device__ __forceinline__ double fixed_sum(const double *v) {
     negs -= (int)sg;
   }
   S += negs;
-#endif
-#if CMG_FXNORM == 1
-  // rounding by the int64 -> FP64 conversion (round to nearest even), then
-  // the exact scaling by 2^(E - 1082) through the exponent field
-  const double d = __ll2double_rn(S);
-  return d == 0.0 ? 0.0 : __hiloint2double(__double2hiint(d) + ((E - 1082) << 20), __double2loint(d));
-#else
-  if (S == 0) return 0.0;
-  const unsigned long long neg = S < 0 ? 1ull : 0ull;
-  const unsigned long long a = neg ? 0ull - (unsigned long long)S : (unsigned long long)S;
-  const int p = 63 - __clzll((long long)a);  // leading bit of |S|, <= 62
-  const int eb = E + p - 59;                 // biased exponent of the sum
-  if (eb <= 0) return ldexp((double)S, E - 1082);  // subnormal sum (never in practice)
-  unsigned long long mant;
-  if (p > 52) {
-    const int r = p - 52;  // 1 .. 10
-#if CMG_FXNORM == 2
-    // round half to even by one biased truncation: adding 2^(r-1) - 1 plus
-    // the last kept bit carries into the kept bits exactly when the dropped
-    // part is above half, or equal to it with the kept part odd
-    const uint32_t lo = (uint32_t)a, hi = (uint32_t)(a >> 32);
-    const unsigned long long b = a + (((1u << (r - 1)) - 1u) + ((__funnelshift_r(lo, hi, r)) & 1u));
-    mant = ((unsigned long long)((uint32_t)(b >> 32) >> r) << 32) |
-           __funnelshift_r((uint32_t)b, (uint32_t)(b >> 32), r);
-#else
-    const unsigned long long q = a >> r, rem = a & ((1ull << r) - 1ull), half = 1ull << (r - 1);
-    mant = q + (unsigned long long)((rem > half) | ((rem == half) & (q & 1ull)));
-#endif
-  } else {
-    mant = a << (52 - p);
-  }
-  // mant carries the leading bit at 2^52 (2^53 after a rounding carry), which
-  // adds the last 1 (or 2) to the exponent field
-  return __longlong_as_double((long long)(((unsigned long long)(eb - 1) << 52) + mant + (neg << 63)));
-#endif
+  return fixed_round(S, E << 20);
 }
 
 // Neighbour sum in the order (-x, +x, -y, +y, -z, +z).  FP32: sequential
-// additions.  FP64 (CMG_NBSUM): 0 = five sequential FP64 additions; 1 = all
-// six in the integer sum; 2 = the x and y neighbours in the integer sum, the
-// two z neighbours by FP64 additions; 3 = five in the integer sum, the last
-// by one FP64 addition (the FP64 and integer pipes share the work).
-// Measured on GB300 (512^3 FP64 colour pass; 256^3 + 3-level FP64 chain on
-// one box): 0 = 0.771 ms; 1 = 0.471 ms; 2 = 0.483 ms, 54.8 ms; 3 = 0.424 ms,
-// 51.6 ms.  Every kernel forms every neighbour sum through this
-// function, so a residual formed right after a colour pass repeats that
-// pass's sums bit for bit.
-#ifndef CMG_NBSUM
-#define CMG_NBSUM 3
-#endif
+// additions.  FP64: the first five in the integer sum, the last by one FP64
+// addition (the FP64 and integer pipes share the work).  Every kernel forms
+// every neighbour sum with these bits, so a residual formed right after a
+// colour pass repeats that pass's sums bit for bit.
 __device__ __forceinline__ float nbsum6(const float v[6]) {
   return ((((v[0] + v[1]) + v[2]) + v[3]) + v[4]) + v[5];
 }
-__device__ __forceinline__ double nbsum6(const double v[6]) {
-#if CMG_NBSUM == 1
-  return fixed_sum<6>(v);
-#elif CMG_NBSUM == 2
-  return (fixed_sum<4>(v) + v[4]) + v[5];
-#elif CMG_NBSUM == 3
-  return fixed_sum<5>(v) + v[5];
-#else
-  return ((((v[0] + v[1]) + v[2]) + v[3]) + v[4]) + v[5];
-#endif
-}
+__device__ __forceinline__ double nbsum6(const double v[6]) { return fixed_sum<5>(v) + v[5]; }
 
-// The neighbour sum of a colour-0 residual cell (CMG_RESID_NB): 0 = nbsum6;
-// 1 = all six in the integer sum.  No colour-0 residual has to repeat a
-// colour pass's sum (only the colour-1 residuals after a colour-1 pass do,
-// and they keep nbsum6), and the residual spends twice the sweep's FP64
-// instructions per cell (the subtraction of phi and the norm or restriction
-// sum), so its best split differs: measured on GB300 (256^3 + 3-level FP64
-// chain, one box), the residual family 11.6 -> 10.9 ms per step with all six
-// in integers.
-#ifndef CMG_RESID_NB
-#define CMG_RESID_NB 1
-#endif
+// The neighbour sum of a colour-0 residual cell: FP64 takes all six in the
+// integer sum.  No colour-0 residual has to repeat a colour pass's sum (only
+// the colour-1 residuals after a colour-1 pass do, and they keep nbsum6), and
+// the residual spends twice the sweep's FP64 instructions per cell (the
+// subtraction of phi and the norm or restriction sum), so its best split
+// differs: measured on GB300 (256^3 + 3-level FP64 chain, one box), the
+// residual family 11.6 -> 10.9 ms per step with all six in integers.
 __device__ __forceinline__ float nbsum6_r0(const float v[6]) { return nbsum6(v); }
-__device__ __forceinline__ double nbsum6_r0(const double v[6]) {
-#if CMG_RESID_NB == 1
-  return fixed_sum<6>(v);
-#else
-  return nbsum6(v);
-#endif
-}
+__device__ __forceinline__ double nbsum6_r0(const double v[6]) { return fixed_sum<6>(v); }
 
 template <typename T>
 __device__ __forceinline__ T fma_t(T a, T b, T c);
@@ -507,100 +450,165 @@ __device__ __forceinline__ void resid_restrict_cell(bool valid, int64_t i, const
   }
 }
 
-// Block index and child bit of the coarse cell at offset e - 1 (e = 0, 1, 2)
-// along one axis from a father cell whose octant bit is cx; the block of 8
-// coarse octs is displaced toward the father's octant.
-__device__ __forceinline__ void axis_cell(int cx, int e, int &a, int &bit) {
-  if (cx == 0) {
-    a = (e == 0);
-    bit = (e != 1);
-  } else {
-    a = (e == 2);
-    bit = (e == 1);
-  }
-}
-
 // Trilinear cell-centred interpolation of a coarse field onto the 8 children
-// of the coarse cell (block octs b, octant cc): per axis weight 3/4 for the
-// father, 1/4 for its neighbour toward the child (Sec. 5.1.1).
+// of a coarse cell: per axis weight 3/4 for the father, 1/4 for its neighbour
+// toward the child (Sec. 5.1.1).
 //
-// CMG_PROLONG_SEP = 1: separably, in units of 1/4 per axis: along x each pair
-// (father, neighbour) becomes 3 a + b in one FMA, then the same along y and
-// along z, giving 64 x the value (weights 27, 9, 3, 1).  A child costs 7 FMAs
-// and the children of an oct share their x and y stages (the 4 colour-1
-// children of an oct 26 FMAs, all 8 of them 38, against 32 and 64 for the
-// weighted eight-term sum); the 64 is divided out exactly (a power of two)
-// in the FMA that adds the correction to phi, or by a multiplication for a
-// plain value.  CMG_PROLONG_SEP = 0: the eight weighted terms in one FMA
-// chain.
-#ifndef CMG_PROLONG_SEP
-#define CMG_PROLONG_SEP 1
-#endif
+// The father is child cc of the block's oct 0; block oct t is displaced along
+// the axes in t toward the father's octant.  On an axis the neighbour toward
+// a child lies in the displaced oct where the child's bit equals the father's,
+// else it is the father's sibling; in both cases its child bit there is the
+// father's flipped.  So with r = c ^ cc ^ 7 (the axes on which child c looks
+// out of the oct), the value child c combines for the axes in t is child
+// cc ^ t of block oct t & r, with weight 3^(3 - |t|) / 64.
+//
+// 64 x the value is formed as one weighted sum.  FP32: separably, 3 a + b in
+// one FMA along x, y and z.  FP64: in integers, as the neighbour sums are
+// (GB300's FP64 pipe ran the separable form's 26 FMAs per oct at 81 % busy
+// while the others idled): significands at the common scale 2^(E - 1078), E
+// the largest biased exponent of the eight (bits under that scale are
+// truncated), times the weights, added as 64-bit integers
+// (|sum| < 64 * 2^56) and rounded once, ties to even: half an ulp plus at
+// most 63/512 ulp of 64 x the largest value, below the three nested roundings
+// of the separable form.  The 64 is divided out exactly (a power of two) in
+// the FMA that adds the correction to phi, or by a multiplication for a
+// plain value.
+// Measured on GB300 (256^3 + 3-level chain, per step): FP64 prolongations
+// 6.73 ms (separable) -> 4.30 ms; FP32 ones 3.51 -> 2.48 ms, from finding the
+// eight values by t & r instead of by selects among 27 places.
 // 3 a + b with one rounding
 template <typename T>
 __device__ __forceinline__ T tri3(T father, T side) {
   return fma_t(T(3), father, side);
 }
-// 64 x the interpolated value of one child from the coarse values around
-// it: vXYZ with 1 = the father's coordinate on that axis, s = its neighbour
-// toward the child.
+// v[t]: the value for the axes in t
 template <typename T>
-__device__ __forceinline__ T interp64(T v111, T vs11, T v1s1, T vss1, T v11s, T vs1s, T v1ss, T vsss) {
-  return tri3(tri3(tri3(v111, vs11), tri3(v1s1, vss1)), tri3(tri3(v11s, vs1s), tri3(v1ss, vsss)));
+__device__ __forceinline__ T interp64_sep(const T v[8]) {
+  return tri3(tri3(tri3(v[0], v[1]), tri3(v[2], v[3])), tri3(tri3(v[4], v[5]), tri3(v[6], v[7])));
+}
+__device__ __forceinline__ float interp64(const float v[8]) { return interp64_sep(v); }
+__device__ __forceinline__ double interp64(const double v[8]) {
+  uint32_t hi[8], lo[8];
+  int e[8], E = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    hi[t] = (uint32_t)__double2hiint(v[t]);
+    lo[t] = (uint32_t)__double2loint(v[t]);
+    e[t] = (int)((hi[t] >> 20) & 0x7FFu);
+    E = max(E, e[t]);
+  }
+  // infinities, NaN and values whose sum could overflow, or all below 2^-960:
+  // FP64 operations; all zero: 0
+  if (E >= 0x7F0 || E < 64) {
+    if (E == 0) {
+      uint32_t nz = 0;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) nz |= (hi[t] & 0x7FFFFFFFu) | lo[t];
+      if (nz == 0) return 0.0;
+    }
+    return interp64_sep(v);
+  }
+  // each significand with its leading bit at bit 63, shifted right by
+  // E - e + 8 (zero and subnormal values vanish); the sign goes with the
+  // weight for the high word, and as a ones' complement for the low one:
+  // -w a = w (~a) - w (2^32 - 1)
+  unsigned long long L = 0;
+  int H = 0, C = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int w = t == 0 ? 27 : t == 7 ? 1 : (t == 3 || t == 5 || t == 6) ? 3 : 9;
+    const uint32_t top = __funnelshift_l(lo[t], hi[t], 11) | 0x80000000u;
+    const unsigned long long a =
+        shr_clamped(((unsigned long long)top << 32) | (lo[t] << 11), (unsigned)(E - e[t] + 8));
+    const int sg = (int)hi[t] >> 31;  // 0 or -1
+    H += (int)(a >> 32) * (w * (sg | 1));
+    L += (unsigned long long)((uint32_t)a ^ (uint32_t)sg) * (unsigned)w;
+    C += sg * w;
+  }
+  const long long S = (long long)L + ((long long)(H + C) << 32) - C;
+  return fixed_round(S, (E + 4) << 20);
 }
 constexpr double kInv64 = 0.015625;
 
-// The 8 children's values (X64 = false) or, with CMG_PROLONG_SEP = 1 and
-// X64 = true, 64 x them.
+// Where a block's coarse values lie: p[t] + 4 oct is the value of child
+// cc ^ t of an oct.
+template <typename T>
+struct CoarseView {
+  const T *p[8];
+};
+template <typename T>
+__device__ __forceinline__ CoarseView<T> coarse_view(const T *cphi, int64_t cn_alloc, int cc) {
+  CoarseView<T> w;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int ch = cc ^ t;
+    w.p[t] = cphi + (cell_parity(ch) ? cn_alloc * 4 : (int64_t)0) + (ch >> 1);
+  }
+  return w;
+}
+
+// 64 x the values of all 8 children (X64) or the values, out[c].
 template <typename T, bool CG, bool X64 = false>
 __device__ __forceinline__ void interp8(const T *cphi, int64_t cn_alloc, const int32_t b[8], int cc, T out[8]) {
-  T v[27];
+  const CoarseView<T> w = coarse_view(cphi, cn_alloc, cc);
 #pragma unroll
-  for (int ez = 0; ez < 3; ++ez)
+  for (int r = 0; r < 8; ++r) {
+    T v[8];
 #pragma unroll
-    for (int ey = 0; ey < 3; ++ey)
+    for (int t = 0; t < 8; ++t) v[t] = ld1<CG>(w.p[t] + (int64_t)b[t & r] * 4);
+    const T z = interp64(v);
+    out[r] = X64 ? z : z * T(kInv64);
+  }
+  // out[r] is child r ^ (cc ^ 7): put them in child order
 #pragma unroll
-      for (int ex = 0; ex < 3; ++ex) {
-        int ax, bx, ay, by, az, bz;
-        axis_cell(cc & 1, ex, ax, bx);
-        axis_cell((cc >> 1) & 1, ey, ay, by);
-        axis_cell((cc >> 2) & 1, ez, az, bz);
-        const int ch = bx | (by << 1) | (bz << 2);
-        const int64_t oct = b[ax | (ay << 1) | (az << 2)];
-        v[ex + 3 * ey + 9 * ez] = ld1<CG>(cphi + ((int64_t)cell_parity(ch) * cn_alloc + oct) * 4 + (ch >> 1));
+  for (int bit = 1; bit < 8; bit <<= 1) {
+    const bool flip = ((cc ^ 7) & bit) != 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (!(c & bit)) {
+        const T x = out[c], y = out[c | bit];
+        out[c] = flip ? y : x;
+        out[c | bit] = flip ? x : y;
       }
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int fx = c & 1, fy = (c >> 1) & 1, fz = (c >> 2) & 1;
-    const int ex1 = fx ? 2 : 0, ey1 = fy ? 2 : 0, ez1 = fz ? 2 : 0;
-#if CMG_PROLONG_SEP
-    const T z = interp64(v[1 + 3 * 1 + 9 * 1], v[ex1 + 3 * 1 + 9 * 1], v[1 + 3 * ey1 + 9 * 1],
-                         v[ex1 + 3 * ey1 + 9 * 1], v[1 + 3 * 1 + 9 * ez1], v[ex1 + 3 * 1 + 9 * ez1],
-                         v[1 + 3 * ey1 + 9 * ez1], v[ex1 + 3 * ey1 + 9 * ez1]);
-    out[c] = X64 ? z : z * T(kInv64);
-#else
-    const T w0 = T(0.75), w1 = T(0.25);
-    T acc = w0 * w0 * w0 * v[1 + 3 * 1 + 9 * 1];
-    acc = fma_t(w1 * w0 * w0, v[ex1 + 3 * 1 + 9 * 1], acc);
-    acc = fma_t(w0 * w1 * w0, v[1 + 3 * ey1 + 9 * 1], acc);
-    acc = fma_t(w1 * w1 * w0, v[ex1 + 3 * ey1 + 9 * 1], acc);
-    acc = fma_t(w0 * w0 * w1, v[1 + 3 * 1 + 9 * ez1], acc);
-    acc = fma_t(w1 * w0 * w1, v[ex1 + 3 * 1 + 9 * ez1], acc);
-    acc = fma_t(w0 * w1 * w1, v[1 + 3 * ey1 + 9 * ez1], acc);
-    acc = fma_t(w1 * w1 * w1, v[ex1 + 3 * ey1 + 9 * ez1], acc);
-    out[c] = acc;
-#endif
   }
 }
 
-// phi + the child's correction as interp8<..., true> gives it
+// 64 x the values of the colour-1 children, out[q] for slot q.
+template <typename T, bool CG>
+__device__ __forceinline__ void interp4_c1(const T *cphi, int64_t cn_alloc, const int32_t b[8], int cc, T out[4]) {
+  const CoarseView<T> w = coarse_view(cphi, cn_alloc, cc);
+  // r = c ^ cc ^ 7 of an odd-parity c has cc's parity: r = R_j, or R_j ^ 7,
+  // with R_j = 0, 3, 5, 6; the slot c >> 1 is then j ^ k
+  const bool odd = cell_parity(cc) != 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int R = plane_cell(0, j);
+    T v[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int32_t o = (t & R) == (t & ~R) ? b[0] : odd ? b[t & ~R] : b[t & R];
+      v[t] = ld1<CG>(w.p[t] + (int64_t)o * 4);
+    }
+    out[j] = interp64(v);
+  }
+  const int k = ((odd ? cc : cc ^ 7) >> 1) & 3;
+#pragma unroll
+  for (int bit = 1; bit < 4; bit <<= 1) {
+    const bool flip = (k & bit) != 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (!(q & bit)) {
+        const T x = out[q], y = out[q | bit];
+        out[q] = flip ? y : x;
+        out[q | bit] = flip ? x : y;
+      }
+  }
+}
+
+// phi + the child's correction, given as 64 x its value
 template <typename T>
 __device__ __forceinline__ T add_corr(T phi, T corr) {
-#if CMG_PROLONG_SEP
   return fma_t(corr, T(kInv64), phi);
-#else
-  return phi + corr;
-#endif
 }
 
 // phi[i] += trilinear interpolation of the coarse correction (active cells).
@@ -628,9 +636,16 @@ __device__ __forceinline__ ProlongIdx prolong_idx(int64_t i, const uint64_t *__r
 template <typename T, bool MASK, bool CG, bool C0D = false>
 __device__ __forceinline__ void prolong_oct_idx(int64_t i, const ProlongIdx &x, int64_t n_alloc, T *phi,
                                                 const T *cphi, int64_t cn_alloc) {
-  T corr[8];
-  interp8<T, CG, true>(cphi, cn_alloc, x.b, x.cc, corr);
   const unsigned m = x.m;
+  T corr[8];
+  if (C0D) {
+    T c1[4];
+    interp4_c1<T, CG>(cphi, cn_alloc, x.b, x.cc, c1);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) corr[plane_cell(1, q)] = c1[q];
+  } else {
+    interp8<T, CG, true>(cphi, cn_alloc, x.b, x.cc, corr);
+  }
 #pragma unroll
   for (int p = C0D ? 1 : 0; p < 2; ++p) {
     T v[4];
@@ -660,30 +675,12 @@ __device__ __forceinline__ void prolong_cell(int64_t i, int c, const uint64_t *_
                                              const uint8_t *__restrict__ active, const T *cphi, int64_t cn_alloc) {
   if (MASK && !((__ldg(active + i) >> c) & 1)) return;
   const int cc = (int)(__ldg(keys + i) & 7);
-  auto val = [&](int ex, int ey, int ez) -> T {
-    int ax, bx, ay, by, az, bz;
-    axis_cell(cc & 1, ex, ax, bx);
-    axis_cell((cc >> 1) & 1, ey, ay, by);
-    axis_cell((cc >> 2) & 1, ez, az, bz);
-    const int ch = bx | (by << 1) | (bz << 2);
-    const int64_t oct = __ldg(blk + (int64_t)(ax | (ay << 1) | (az << 2)) * n + i);
-    return ld1<CG>(cphi + ((int64_t)cell_parity(ch) * cn_alloc + oct) * 4 + (ch >> 1));
-  };
-  const int ex1 = (c & 1) ? 2 : 0, ey1 = ((c >> 1) & 1) ? 2 : 0, ez1 = ((c >> 2) & 1) ? 2 : 0;
-#if CMG_PROLONG_SEP
-  const T acc = interp64(val(1, 1, 1), val(ex1, 1, 1), val(1, ey1, 1), val(ex1, ey1, 1), val(1, 1, ez1),
-                         val(ex1, 1, ez1), val(1, ey1, ez1), val(ex1, ey1, ez1));
-#else
-  const T w0 = T(0.75), w1 = T(0.25);
-  T acc = w0 * w0 * w0 * val(1, 1, 1);
-  acc = fma_t(w1 * w0 * w0, val(ex1, 1, 1), acc);
-  acc = fma_t(w0 * w1 * w0, val(1, ey1, 1), acc);
-  acc = fma_t(w1 * w1 * w0, val(ex1, ey1, 1), acc);
-  acc = fma_t(w0 * w0 * w1, val(1, 1, ez1), acc);
-  acc = fma_t(w1 * w0 * w1, val(ex1, 1, ez1), acc);
-  acc = fma_t(w0 * w1 * w1, val(1, ey1, ez1), acc);
-  acc = fma_t(w1 * w1 * w1, val(ex1, ey1, ez1), acc);
-#endif
+  const CoarseView<T> w = coarse_view(cphi, cn_alloc, cc);
+  const int r = c ^ cc ^ 7;
+  T v[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) v[t] = ld1<CG>(w.p[t] + (int64_t)__ldg(blk + (int64_t)(t & r) * n + i) * 4);
+  const T acc = interp64(v);
   T *dst = phi + ((int64_t)cell_parity(c) * n_alloc + i) * 4 + (c >> 1);
   *dst = add_corr(ld1<CG>(dst), acc);
 }
