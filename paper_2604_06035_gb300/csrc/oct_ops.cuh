@@ -24,6 +24,21 @@ __device__ __forceinline__ T ld1(const T *p) {
   if constexpr (CG) return __ldcg(p); else return *p;
 }
 
+// The four values of one plane of an oct in one access (16 bytes FP32, 32
+// bytes FP64; oct arrays start on 32-byte boundaries).
+__device__ __forceinline__ void load_oct(const double *p, double v[4]) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void load_oct(const float *p, float v[4]) {
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+               : "l"(p)
+               : "memory");
+}
+
 template <bool CG>
 __device__ __forceinline__ void load4(const double *p, double v[4]) {
   const double2 a = ldv<CG>(reinterpret_cast<const double2 *>(p));
@@ -218,6 +233,14 @@ __device__ __forceinline__ void sweep_oct_idx(int64_t i, const SweepIdx &x, cons
     load4<CG>(src + i * 4, own);
     const int32_t *nb = x.nb;
     const T inv6 = T(1) / T(6);
+    // whole neighbour octs, two of their values used each: fewer, wider loads
+    // than one per value (256^3 + 3-level chains: FP32 passes 16.95 -> 16.35
+    // ms per step, FP64 ones 26.96 -> 26.52)
+    T nv[6][4];
+    if (!CG) {
+#pragma unroll
+      for (int d = 0; d < 6; ++d) load_oct(src + (int64_t)nb[d] * 4, nv[d]);
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int c = plane_cell(P, q);
@@ -225,7 +248,9 @@ __device__ __forceinline__ void sweep_oct_idx(int64_t i, const SweepIdx &x, cons
 #pragma unroll
       for (int d = 0; d < 6; ++d) {
         const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
-        v[d] = (((c >> a) & 1) != side) ? own[c2 >> 1] : ld1<CG>(src + (int64_t)nb[d] * 4 + (c2 >> 1));
+        if (((c >> a) & 1) != side) v[d] = own[c2 >> 1];
+        else if (!CG) v[d] = nv[d][c2 >> 1];
+        else v[d] = ld1<CG>(src + (int64_t)nb[d] * 4 + (c2 >> 1));
       }
       out[q] = fma_t(nbsum6(v), inv6, gv[q]);
     }
