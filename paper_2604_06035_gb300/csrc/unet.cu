@@ -182,6 +182,11 @@ struct WgradGeom {
   static constexpr int kHaloPlane = (kRows * 16 + 127) / 128 * 128 + 64;
   static constexpr int kDoutPlane = kVox * 16 + 1024 / COUT;
   static constexpr int kStage = (2 * kHaloPlane + (COUT / 8) * kDoutPlane + 127) / 128 * 128;
+  // The tensor cores truncate as they accumulate, an error that grows with the
+  // number of MMAs in a row: with 16 output channels (the D grid: the most
+  // bricks per block) the sums move to a second set of registers, by FP32
+  // additions, every kFlush bricks.
+  static constexpr int kFlush = COUT == 16 ? 16 : 0;
   static constexpr int kStages = COUT == 64 ? 2 : 3;  // what two blocks per SM leave room for
   static constexpr int kChunks = kVox / 16 / KW;       // 16-voxel chunks per warp, whole z slices
   static constexpr int kRed = 27 * 16 * COUT * 4;
@@ -235,6 +240,26 @@ __global__ void __launch_bounds__(WgradGeom<COUT, BX, BY, BZ>::kThreads, WgradGe
   };
 
   float acc[9][NM][2][4], accb[NM][4];
+  constexpr int kTot = G::kFlush ? 9 * NM * 8 + NM * 4 : 1;
+  float tot[kTot];
+#pragma unroll
+  for (int k = 0; k < kTot; ++k) tot[k] = 0.f;
+  auto flush = [&]() {
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+#pragma unroll
+      for (int k = 0; k < 72; ++k) {
+        float &x = acc[k / 8][m][(k / 4) % 2][k % 4];
+        tot[m * 72 + k] += x;
+        x = 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        tot[NM * 72 + m * 4 + k] += accb[m][k];
+        accb[m][k] = 0.f;
+      }
+    }
+  };
 #pragma unroll
   for (int m = 0; m < NM; ++m) {
 #pragma unroll
@@ -249,7 +274,7 @@ __global__ void __launch_bounds__(WgradGeom<COUT, BX, BY, BZ>::kThreads, WgradGe
   const uint32_t lane_a = ahalf * G::kDoutPlane + (kw * G::kChunks * 16 + ak) * 16;
   const uint32_t lane_b = bhalf * G::kHaloPlane +
                           ((kw * G::kChunks * 16 / (BX * BY) + dz) * (G::HX * G::HY) + (bk / BX) * G::HX + bk % BX) * 16;
-  int buf = 0;
+  int buf = 0, since = 0;
 #pragma unroll
   for (int k = 0; k < G::kStages - 1; ++k) {
     if (blockIdx.x + k * (int)gridDim.x < nbricks) stage(blockIdx.x + k * gridDim.x, k);
@@ -286,6 +311,22 @@ __global__ void __launch_bounds__(WgradGeom<COUT, BX, BY, BZ>::kThreads, WgradGe
 #pragma unroll
         for (int m = 0; m < NM; ++m) mma16816(accb[m], a[m][0], a[m][1], a[m][2], a[m][3], kOnes, kOnes);
       }
+    }
+    if constexpr (G::kFlush > 0) {
+      if (++since == G::kFlush) {
+        flush();
+        since = 0;
+      }
+    }
+  }
+  if constexpr (G::kFlush > 0) {
+    flush();
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+#pragma unroll
+      for (int k = 0; k < 72; ++k) acc[k / 8][m][(k / 4) % 2][k % 4] = tot[m * 72 + k];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) accb[m][k] = tot[NM * 72 + m * 4 + k];
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
