@@ -29,12 +29,22 @@ T *DeviceBuffers::alloc(int64_t count, bool zero, cudaStream_t s) {
   const size_t bytes = sizeof(T) * (size_t)(count > 0 ? count : 1);
   if (g_alloc_countdown.load() > 0 && g_alloc_countdown.fetch_sub(1) == 1)
     throw Error(CMG_ERR_OOM, "injected allocation failure (" + std::to_string(bytes) + " bytes)");
-  cudaError_t e = cudaMalloc(&p, bytes);
+  // not into a stream capture of the caller's: the memory would be the graph's
+  bool async = pool != nullptr;
+  if (async) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+      cudaGetLastError();
+      async = false;
+    }
+    async = async && cap == cudaStreamCaptureStatusNone;
+  }
+  cudaError_t e = async ? cudaMallocFromPoolAsync(&p, bytes, pool, stream) : cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    throw Error(CMG_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
+    throw Error(CMG_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
   }
-  ptrs.push_back(p);
+  (async ? pooled : ptrs).push_back(p);
   if (zero) CMG_CUDA(cudaMemsetAsync(p, 0, bytes, s));
   return static_cast<T *>(p);
 }
@@ -42,6 +52,54 @@ T *DeviceBuffers::alloc(int64_t count, bool zero, cudaStream_t s) {
 void DeviceBuffers::release() {
   for (void *p : ptrs) cudaFree(p);
   ptrs.clear();
+  for (void *p : pooled)
+    if (cudaFreeAsync(p, stream) != cudaSuccess) {  // the stream is gone
+      cudaGetLastError();
+      cudaFree(p);
+    }
+  // the pool gives back what it does not keep at this wait
+  if (!pooled.empty()) cudaStreamSynchronize(stream);
+  pooled.clear();
+}
+
+LevelMemory::LevelMemory(int device) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  CMG_CUDA(cudaMemPoolCreate(&pool, &props));
+  uint64_t kept = kKept;
+  CMG_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &kept));
+}
+
+LevelMemory::~LevelMemory() {
+  for (void *p : pinned) cudaFreeHost(p);
+  if (pool) cudaMemPoolDestroy(pool);
+}
+
+void *LevelMemory::take_pinned() {
+  {
+    std::lock_guard<std::mutex> lock(m);
+    if (!pinned.empty()) {
+      void *p = pinned.back();
+      pinned.pop_back();
+      return p;
+    }
+  }
+  void *p = nullptr;
+  CMG_CUDA(cudaMallocHost(&p, kPinnedBytes));
+  return p;
+}
+
+void LevelMemory::give_pinned(void *p) {
+  {
+    std::lock_guard<std::mutex> lock(m);
+    if (pinned.size() < kPinnedKept) {
+      pinned.push_back(p);
+      return;
+    }
+  }
+  cudaFreeHost(p);
 }
 
 template uint64_t *DeviceBuffers::alloc<uint64_t>(int64_t, bool, cudaStream_t);
@@ -328,35 +386,29 @@ __global__ void k_parent_emit(const K *__restrict__ keys, int64_t n, const int32
   if (flag[i]) ckeys[pos[i]] = KeyOps<K>::parent(keys[i]);
 }
 
-// Coarse cell active iff a fully active fine oct refines it (pull).
-template <class K>
-__global__ void k_coarse_active(const K *__restrict__ ckeys, int64_t cn, const K *__restrict__ f_ht_keys,
-                                const int32_t *__restrict__ f_ht_vals, uint64_t f_mask,
-                                const uint8_t *__restrict__ f_active, bool f_all_active,
-                                uint8_t *__restrict__ cactive) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= cn) return;
-  const K k = ckeys[p];
-  uint8_t m = 0;
-  for (int c = 0; c < 8; ++c) {
-    const int32_t i = ht_find_k(f_ht_keys, f_ht_vals, f_mask, KeyOps<K>::child(k, c));
-    if (i >= 0 && (f_all_active || f_active[i] == 0xFF)) m |= (uint8_t)(1u << c);
-  }
-  cactive[p] = m;
-}
-
+// Father cells and interpolation blocks of a level's octs in the coarser
+// one, and the coarse cells' activity: a coarse cell is active iff a fully
+// active fine oct refines it, so each such oct sets its father's bit (cactive
+// starts at zero; four octs' masks share a word).  One pass: looking the 8
+// possible children of every coarse oct up in the fine table instead took as
+// long as everything else here (28 us of a 178k-oct level's build).
 template <class K>
 __global__ void k_father_and_block(const K *__restrict__ keys, const uint8_t *__restrict__ active, bool all_active,
                                    int64_t n, uint64_t cnpd, int pmask, const K *__restrict__ c_ht_keys,
                                    const int32_t *__restrict__ c_ht_vals, uint64_t c_mask, int32_t c_zero,
-                                   int32_t *__restrict__ father, int32_t *__restrict__ blk) {
+                                   int32_t *__restrict__ father, int32_t *__restrict__ blk,
+                                   uint32_t *__restrict__ cactive) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const K k = keys[i];
   int32_t fa = -1;
   if (all_active || active[i] == 0xFF) {
     const int32_t p = ht_find_k(c_ht_keys, c_ht_vals, c_mask, KeyOps<K>::parent(k));
-    if (p >= 0) fa = p * 8 + (int32_t)KeyOps<K>::octant(k);
+    if (p >= 0) {
+      const int oc = (int)KeyOps<K>::octant(k);
+      fa = p * 8 + oc;
+      atomicOr(cactive + (p >> 2), 1u << (8 * (p & 3) + oc));
+    }
   }
   father[i] = fa;
   int32_t b[8];
@@ -422,18 +474,19 @@ __global__ void k_active_bytes(const uint8_t *__restrict__ active, bool all_acti
 
 // ------------------------------------------------------------ host helpers
 
-int read_error(cmg_ctx *ctx) {
-  CMG_CUDA(cudaMemcpyAsync(ctx->h_pinned, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+// One wait for the device error flag and the build's counters (d_err[4] ..
+// [6]); throws on an error.
+const char *status_text(int e);
+enum { kMissing = 0, kGhosts = 1, kParents = 2 };
+int32_t read_counter(cmg_ctx *ctx, int which) {
+  CMG_CUDA(cudaMemcpyAsync(ctx->h_pinned, ctx->d_err, 8 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CMG_CUDA(cudaStreamSynchronize(ctx->stream));
   const int e = ctx->h_pinned[0];
-  if (e != 0) CMG_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
-  return e;
-}
-
-int32_t read_i32(cmg_ctx *ctx, const int32_t *d) {
-  CMG_CUDA(cudaMemcpyAsync(ctx->h_pinned + 1, d, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-  CMG_CUDA(cudaStreamSynchronize(ctx->stream));
-  return ctx->h_pinned[1];
+  if (e != 0) {
+    CMG_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
+    throw Error(e, status_text(e));
+  }
+  return ctx->h_pinned[4 + which];
 }
 
 const char *status_text(int e) {
@@ -489,21 +542,19 @@ void build_level_t(cmg_level *L, const K *keys, cmg_mem mem) {
   if (top.n > 0)
     CMG_CUDA(cudaMemcpyAsync(tkeys, keys, sizeof(K) * top.n,
                              mem == CMG_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
-  CMG_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), s));
+  CMG_CUDA(cudaMemsetAsync(ctx->d_err, 0, 8 * sizeof(int), s));
+  int32_t *d_cnt = ctx->d_err + 4;
   build_hash<K>(L, top, npd);
   low_words<K>(L, top);
-  int e = read_error(ctx);
-  if (e) throw Error(e, status_text(e));
   const K *ttab = LevelKeys<K>::table(top);
 
   // neighbour cache; INT_MIN marks "missing" until ghosts are assigned
-  int32_t *d_cnt = L->mem.alloc<int32_t>(4, true, s);
   top.nbr = L->mem.alloc<int32_t>(6 * top.n);
   if (top.n > 0)
     k_neighbors<K><<<blocks_for(top.n), kThreads, 0, s>>>(tkeys, top.n, npd, L->pmask, ttab, top.ht_vals,
-                                                           (uint64_t)top.cap - 1, INT_MIN, top.nbr, d_cnt);
+                                                           (uint64_t)top.cap - 1, INT_MIN, top.nbr, d_cnt + kMissing);
   CMG_CUDA(cudaGetLastError());
-  const int32_t n_missing = read_i32(ctx, d_cnt);
+  const int32_t n_missing = read_counter(ctx, kMissing);
 
   top.n_ghost = 0;
   if (L->parent && n_missing > 0) {
@@ -513,11 +564,10 @@ void build_level_t(cmg_level *L, const K *keys, cmg_mem mem) {
     CMG_CUDA(cudaMemsetAsync(g_keys, 0xFF, sizeof(K) * gcap, s));
     K *gk = L->mem.alloc<K>(n_missing);
     k_ghost_insert<K><<<blocks_for(top.n), kThreads, 0, s>>>(tkeys, top.n, npd, L->pmask, top.nbr, INT_MIN, g_keys,
-                                                              g_vals, (uint64_t)gcap - 1, d_cnt + 1, gk, ctx->d_err);
+                                                              g_vals, (uint64_t)gcap - 1, d_cnt + kGhosts, gk,
+                                                              ctx->d_err);
     CMG_CUDA(cudaGetLastError());
-    e = read_error(ctx);
-    if (e) throw Error(e, status_text(e));
-    top.n_ghost = read_i32(ctx, d_cnt + 1);
+    top.n_ghost = read_counter(ctx, kGhosts);
     if constexpr (sizeof(K) == 16) {
       L->ghost_keys128 = gk;
       L->ghost_keys = L->mem.alloc<uint64_t>(top.n_ghost > 0 ? top.n_ghost : 1);
@@ -536,8 +586,6 @@ void build_level_t(cmg_level *L, const K *keys, cmg_mem mem) {
         gk, top.n_ghost, L->ghost_mask, octs_per_dim(L, L->lev - 1), L->pmask, LevelKeys<K>::table(pg), pg.ht_vals,
         (uint64_t)pg.cap - 1, (int32_t)(pg.n_alloc - 1), L->ghost_blk, ctx->d_err);
     CMG_CUDA(cudaGetLastError());
-    e = read_error(ctx);
-    if (e) throw Error(e, status_text(e));
   }
   top.n_alloc = top.n + top.n_ghost + 1;
   // remaining missing neighbours (no parent): the zero oct
@@ -571,8 +619,8 @@ void build_level_t(cmg_level *L, const K *keys, cmg_mem mem) {
                                                             t_min, (uint64_t)tcap - 1, flag);
     }
     CMG_CUDA(cudaGetLastError());
-    scan_exclusive(flag, pos, n, d_cnt + 2, scratch, scratch_n, s);
-    const int32_t np = read_i32(ctx, d_cnt + 2);
+    scan_exclusive(flag, pos, n, d_cnt + kParents, scratch, scratch_n, s);
+    const int32_t np = read_counter(ctx, kParents);  // and the errors of the steps before
     if (np == 0) break;
     L->mg.emplace_back();
     MgLev &c = L->mg.back();
@@ -594,23 +642,20 @@ void build_level_t(cmg_level *L, const K *keys, cmg_mem mem) {
     c.nbr = L->mem.alloc<int32_t>(6 * np);
     k_neighbors<K><<<blocks_for(np), kThreads, 0, s>>>(ckeys, np, cnpd, L->pmask, ctab, c.ht_vals,
                                                         (uint64_t)c.cap - 1, (int32_t)np, c.nbr, nullptr);
-    c.active = L->mem.alloc<uint8_t>(np);
-    k_coarse_active<K><<<blocks_for(np), kThreads, 0, s>>>(ckeys, np, LevelKeys<K>::table(f), f.ht_vals,
-                                                            (uint64_t)f.cap - 1, f.active, f.all_active, c.active);
+    c.active = L->mem.alloc<uint8_t>((np + 3) / 4 * 4, true, s);
     f.father = L->mem.alloc<int32_t>(n);
     f.blk = L->mem.alloc<int32_t>(8 * n);
     k_father_and_block<K><<<blocks_for(n), kThreads, 0, s>>>(LevelKeys<K>::keys(f), f.active, f.all_active, n, cnpd,
                                                               L->pmask, ctab, c.ht_vals, (uint64_t)c.cap - 1,
-                                                              (int32_t)np, f.father, f.blk);
+                                                              (int32_t)np, f.father, f.blk,
+                                                              reinterpret_cast<uint32_t *>(c.active));
     CMG_CUDA(cudaGetLastError());
     c.phi = L->mem.alloc<double>(8 * c.n_alloc, true, s);
     c.g = L->mem.alloc<double>(8 * c.n, true, s);
-    e = read_error(ctx);
-    if (e) throw Error(e, status_text(e));
   }
   const MgLev &last = L->mg.back();
   L->exact_coarse = L->periodic_full && last.lev == 1 && L->nx == 1 && last.n == 1;
-  CMG_CUDA(cudaStreamSynchronize(s));
+  (void)read_counter(ctx, kParents);
 }
 
 }  // namespace

@@ -209,6 +209,7 @@ int cmg_ctx_create(int device, void *stream, cmg_ctx **out) {
     c->stream = static_cast<cudaStream_t>(stream);
     try {
       CMG_CUDA(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device));
+      c->level_memory = std::make_shared<cmg::LevelMemory>(device);
       CMG_CUDA(cudaMalloc(&c->d_err, 64));
       CMG_CUDA(cudaMemsetAsync(c->d_err, 0, 64, c->stream));
       CMG_CUDA(cudaMallocHost(&c->h_pinned, 64));
@@ -369,6 +370,9 @@ int level_build(cmg_ctx *ctx, int level, int nx, int periodic_mask, const void *
     L->n = n_octs;
     L->parent = parent;
     L->key_bits = key_bits;
+    L->memory = ctx->level_memory;
+    L->mem.pool = L->memory->pool;
+    L->mem.stream = ctx->stream;
     const uint64_t npd = (uint64_t)nx << (level - 1);
     L->periodic_full = parent == nullptr && periodic_mask == 7 && npd <= 2048 && (uint64_t)n_octs == npd * npd * npd;
     try {
@@ -414,7 +418,7 @@ int cmg_level_destroy(cmg_level *lvl) {
   cudaSetDevice(lvl->device);  // the level's own copies: no use of its context
   cudaStreamSynchronize(lvl->stream);
   cmg::destroy_graphs(lvl);
-  if (lvl->h_ctrl) cudaFreeHost(lvl->h_ctrl);
+  if (lvl->h_ctrl) lvl->memory->give_pinned(lvl->h_ctrl);
   if (lvl->ev_start) cudaEventDestroy(lvl->ev_start);
   if (lvl->ev_end) cudaEventDestroy(lvl->ev_end);
   lvl->mem.release();
