@@ -14,8 +14,9 @@ namespace cmg {
 namespace {
 
 // Deterministic block sum of one double per thread -> partials[blockIdx.x].
+template <int THREADS = kThreads>
 __device__ void block_sum_to(double v, double *partials) {
-  __shared__ double ws[kThreads / 32];
+  __shared__ double ws[THREADS / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
@@ -40,6 +41,8 @@ template <typename T>
 constexpr bool kPreloadIdx = sizeof(T) == 4;
 constexpr int64_t kPreloadSweepOcts = int64_t(1) << 20;
 
+constexpr int kCellThreads = 128;
+
 template <typename T, int P, bool ZERO, bool MASK, bool PRE>
 __global__ void __launch_bounds__(kThreads) k_sweep(const int32_t *__restrict__ nbr, const T *__restrict__ src,
                                                    T *__restrict__ dst, const T *__restrict__ g,
@@ -56,6 +59,69 @@ __global__ void __launch_bounds__(kThreads) k_sweep(const int32_t *__restrict__ 
     if (i >= n) return;
     dev::sweep_oct<T, P, ZERO, MASK, false>(i, nbr, src, dst, g, active, n);
   }
+}
+
+// FP64 operations with one thread per cell (four per oct).
+template <int P, bool ZERO, bool MASK>
+__global__ void __launch_bounds__(kCellThreads) k_sweep_cell(const int32_t *__restrict__ nbr,
+                                                            const double *__restrict__ src, double *__restrict__ dst,
+                                                            const double *__restrict__ g,
+                                                            const uint8_t *__restrict__ active, int64_t n) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_enter();
+  if (t >= 4 * n) return;
+  dev::sweep_cell<double, P, ZERO, MASK, false>(t >> 2, (int)(t & 3), nbr, src, dst, g, active, n);
+}
+
+// Restriction of the colour-0 residuals (the colour-1 ones are zero): the
+// four lanes of an oct hand theirs to the first, which adds them in resid_oct's
+// order.  Every thread of a warp runs it.
+template <bool MASK>
+__global__ void __launch_bounds__(kCellThreads)
+    k_restrict_cell(const int32_t *__restrict__ nbr, const double *__restrict__ phi, const double *__restrict__ g,
+                    const uint8_t *__restrict__ active, int64_t n, int64_t n_alloc,
+                    const int32_t *__restrict__ father, double *__restrict__ cg, double *__restrict__ cphi, int64_t cn,
+                    int64_t cn_alloc, int zero_cphi) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_enter();
+  const int64_t i = t >> 2;
+  const bool on = i < n;
+  const double dv = on ? dev::resid_c0_cell<MASK>(i, (int)(t & 3), nbr, phi, g, active, n, n_alloc) : 0.0;
+  const int base = (int)(threadIdx.x & 31) & ~3;
+  double rsum = 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) rsum += __shfl_sync(0xFFFFFFFFu, dv, base + j);
+  if (!on || (t & 3)) return;
+  const int32_t fa = __ldg(father + i);
+  if (fa < 0) return;
+  const int64_t pc = fa >> 3;
+  const int cc = fa & 7;
+  cg[((int64_t)cell_parity(cc) * cn + pc) * 4 + (cc >> 1)] = 0.5 * rsum;
+  if (zero_cphi) cphi[((int64_t)cell_parity(cc) * cn_alloc + pc) * 4 + (cc >> 1)] = 0.0;
+}
+
+// Sum of the colour-0 residuals' squares, per block of 256 octs as in k_resid.
+template <bool MASK>
+__global__ void __launch_bounds__(4 * kThreads)
+    k_norm_cell(const int32_t *__restrict__ nbr, const double *__restrict__ phi, const double *__restrict__ g,
+                const uint8_t *__restrict__ active, int64_t n, int64_t n_alloc, double *__restrict__ partials) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_enter();
+  const double dv = (t >> 2) < n ? dev::resid_c0_cell<MASK>(t >> 2, (int)(t & 3), nbr, phi, g, active, n, n_alloc) : 0.0;
+  block_sum_to<4 * kThreads>(dv * dv, partials);
+}
+
+// Prolongation before a colour-0 pass: the colour-1 cells only.
+template <bool MASK>
+__global__ void __launch_bounds__(kCellThreads)
+    k_prolong_cell(const uint64_t *__restrict__ keys, const int32_t *__restrict__ blk, int64_t n, int64_t n_alloc,
+                   double *__restrict__ phi, const uint8_t *__restrict__ active, const double *__restrict__ cphi,
+                   int64_t cn_alloc) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_enter();
+  if (t >= 4 * n) return;
+  dev::prolong_cell<double, MASK, false>(t >> 2, plane_cell(1, (int)(t & 3)), keys, blk, n, n_alloc, phi, active, cphi,
+                                         cn_alloc);
 }
 
 template <typename T, bool NORM, bool RESTRICT, bool EMIT, bool ROUT, bool ZPHI, bool C1Z = false>

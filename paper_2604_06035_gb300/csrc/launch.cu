@@ -8,6 +8,18 @@
 
 namespace cmg {
 
+// Small FP64 levels run one thread per cell instead of one per oct: four
+// times the warps, each with a quarter of the oct's FP64 instructions (which
+// issue once per ~64 clocks and sub-partition), so that a launch which does
+// not fill the GPU ends sooner; above, the per-cell loads and index reads
+// cost more.  Residuals and prolongations: up to where 4 n threads fill the
+// 152 SMs about once; colour passes gain further.  Measured (GB300, per
+// solve): 32^3 0.959 -> 0.873 ms, 64^3 two-level CG 2.34 -> 2.27 ms; 128^3
+// two-level 4.13 -> 4.06 ms with passes per cell up to its 179k-oct level,
+// 4.16 ms with its residuals and prolongations too, 4.62 ms with everything
+// on the 262k-oct level.
+constexpr int64_t kCellOcts = 40000, kCellSweepOcts = 200000;
+
 // ------------------------------------------------------------ launchers
 // Algorithmic work per launch (for the profile): bytes are the minimum
 // traffic of the operation with perfect reuse, flops its floating-point
@@ -30,9 +42,17 @@ void sweep(cmg_level *L, int m, bool zero_init) {
   const double nbr_bytes = 12.0 * (double)g.n;
   const double full_bytes = 3.0 * u * sizeof(T) + nbr_bytes, full_flops = 7.0 * u;
   const bool pre = kPreloadIdx<T> && g.n <= kPreloadSweepOcts;
+  const bool per_cell = sizeof(T) == 8 && g.n <= kCellSweepOcts;
 #define CMG_SWEEP(P, Z, M)                                                                                  \
   do {                                                                                                      \
     LaunchScope ls(L->ctx, cls, (Z) ? 2.0 * u * sizeof(T) + nbr_bytes : full_bytes, (Z) ? 0.0 : full_flops); \
+    if constexpr (sizeof(T) == 8) {                                                                         \
+      if (per_cell) {                                                                                       \
+        launch_k(k_sweep_cell<P, Z, M>, blocks_for(4 * g.n, kCellThreads), kCellThreads, s, g.nbr,          \
+                 phi + (1 - P) * st, phi + P * st, gg + P * g.n * 4, g.active, g.n);                        \
+        break;                                                                                              \
+      }                                                                                                     \
+    }                                                                                                       \
     if (pre)                                                                                                \
       launch_k(k_sweep<T, P, Z, M, kPreloadIdx<T>>, nb, kThreads, s, g.nbr, phi + (1 - P) * st, phi + P * st, \
                gg + P * g.n * 4, g.active, g.n);                                                            \
@@ -77,7 +97,22 @@ void resid_restrict(cmg_level *L, int m, bool restrict_to_coarse, bool norm, boo
   const int cls = sizeof(T) == 8 ? K_RESID64 : K_RESID32;
   if (g.n > 0) {
     LaunchScope ls(L->ctx, cls, bytes, flops);
-    if (restrict_to_coarse && !norm && !emit_scale && c1_swept)
+    bool done = false;
+    if constexpr (sizeof(T) == 8) {
+      if (c1_swept && !emit_scale && g.n <= kCellOcts && restrict_to_coarse != norm) {
+        if (restrict_to_coarse)
+          launch_k(act ? k_restrict_cell<true> : k_restrict_cell<false>, blocks_for(4 * g.n, kCellThreads),
+                   kCellThreads, s, g.nbr, g.phi, g.g, act, g.n, g.n_alloc, g.father, cg, cphi, cn, cna,
+                   (int)zero_coarse_phi);
+        else
+          launch_k(act ? k_norm_cell<true> : k_norm_cell<false>, nb, 4 * kThreads, s, g.nbr, g.phi, g.g, act, g.n,
+                   g.n_alloc, L->partials);
+        done = true;
+      }
+    }
+    if (done)
+      ;
+    else if (restrict_to_coarse && !norm && !emit_scale && c1_swept)
       launch_k(k_resid<T, false, true, false, false, false, true>, nb, kThreads, s,
           g.nbr, phi_of<T>(g), g_of<T>(g), act, g.n, g.n_alloc, g.father, cg, cphi, cn, cna, zero_coarse_phi,
           nullptr, nullptr, nullptr, nullptr, 0.0);
@@ -170,6 +205,14 @@ void prolong(cmg_level *L, int m, bool c0_dead) {
   LaunchScope ls(L->ctx, sizeof(T) == 8 ? K_PROLONG64 : K_PROLONG32,
                  g.n * (c0_dead ? 9.0 : 17.0) * sizeof(T), g.n * (c0_dead ? 64.0 : 128.0));
   const unsigned nb = blocks_for(g.n);
+  if constexpr (sizeof(T) == 8) {
+    if (c0_dead && g.n <= kCellOcts) {
+      launch_k(g.all_active ? k_prolong_cell<false> : k_prolong_cell<true>, blocks_for(4 * g.n, kCellThreads),
+               kCellThreads, s, g.keys, g.blk, g.n, g.n_alloc, g.phi, g.active, c.phi, c.n_alloc);
+      CMG_CUDA(cudaGetLastError());
+      return;
+    }
+  }
   if (g.all_active && c0_dead)
     launch_k(k_prolong<T, false, true>, nb, kThreads, s, g.keys, g.blk, g.n, g.n_alloc, phi_of<T>(g), g.active,
              phi_of<T>(c), c.n_alloc);

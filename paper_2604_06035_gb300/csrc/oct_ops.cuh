@@ -475,6 +475,25 @@ __device__ __forceinline__ void resid_restrict_cell(bool valid, int64_t i, const
   }
 }
 
+// resid_oct<..., C1Z = true> with four threads per oct: the residual of colour
+// 0 cell q of oct i (d-units), the same sum and operations.
+template <bool MASK>
+__device__ __forceinline__ double resid_c0_cell(int64_t i, int q, const int32_t *__restrict__ nbr, const double *phi,
+                                                const double *g, const uint8_t *__restrict__ active, int64_t n,
+                                                int64_t n_alloc) {
+  const int c = plane_cell(0, q);
+  const double pv = phi[i * 4 + q], gv = g[i * 4 + q];
+  double v[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
+    const int64_t o = (((c >> a) & 1) != side) ? i : (int64_t)__ldg(nbr + d * n + i);
+    v[d] = phi[(n_alloc + o) * 4 + (c2 >> 1)];
+  }
+  const double dv = fma(nbsum6_r0(v), 1.0 / 6.0, gv) - pv;
+  return MASK && !((__ldg(active + i) >> c) & 1) ? 0.0 : dv;
+}
+
 // Trilinear cell-centred interpolation of a coarse field onto the 8 children
 // of a coarse cell: per axis weight 3/4 for the father, 1/4 for its neighbour
 // toward the child (Sec. 5.1.1).
