@@ -231,58 +231,130 @@ __global__ void k_wht(const T *__restrict__ g, T *__restrict__ phi, int64_t n_al
   dev::wht_solve_warp<T, T, false>(g, phi, n_alloc, h);
 }
 
-__global__ void k_set_density(const double *__restrict__ rho, int64_t n, double rho_bar, double scale,
-                              double *__restrict__ g) {
+// The layout kernels below take one oct per thread: its 8 values in 16-byte
+// accesses, which moves a 256^3 level's field at about twice the rate of one
+// value per thread.  WIDE = false: the caller's array does not start on a
+// 16-byte boundary and is accessed value by value.
+template <bool WIDE, typename T>
+__device__ __forceinline__ void load8(const T *p, T v[8]) {
+  if (!WIDE) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = p[k];
+    return;
+  }
+  T a[4], b[4];
+  dev::load4<false>(p, a);
+  dev::load4<false>(p + 4, b);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = a[k];
+    v[k + 4] = b[k];
+  }
+}
+template <bool WIDE, typename T>
+__device__ __forceinline__ void store8(T *p, const T v[8]) {
+  if (!WIDE) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) p[k] = v[k];
+    return;
+  }
+  dev::store4(p, v);
+  dev::store4(p + 4, v + 4);
+}
+// the plane's four values of an oct's eight (child order), and back
+template <typename T>
+__device__ __forceinline__ void to_plane(const T v[8], int p, T q4[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) q4[q] = p == 0 ? v[plane_cell(0, q)] : v[plane_cell(1, q)];
+}
+
+template <bool WIDE>
+__global__ void __launch_bounds__(kThreads) k_set_density(const double *__restrict__ rho, int64_t n, double rho_bar,
+                                                         double scale, double *__restrict__ g) {
   pdl_enter();
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 8 * n) return;
-  const int64_t i = t >> 3;
-  const int c = (int)(t & 7);
-  g[((int64_t)cell_parity(c) * n + i) * 4 + (c >> 1)] = scale * (rho[t] - rho_bar);
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double v[8], w[4];
+  load8<WIDE>(rho + i * 8, v);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) v[c] = scale * (v[c] - rho_bar);
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    to_plane(v, p, w);
+    dev::store4(g + (p * n + i) * 4, w);
+  }
 }
 
 // oct-major [n][8] <-> planar [2][stride][4], with a scale factor
-template <typename S, typename D>
-__global__ void k_pack(const S *__restrict__ in, int64_t n, int64_t stride, double scale, D *__restrict__ out) {
-  pdl_enter();
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 8 * n) return;
-  const int64_t i = t >> 3;
-  const int c = (int)(t & 7);
-  out[((int64_t)cell_parity(c) * stride + i) * 4 + (c >> 1)] = (D)(scale * (double)in[t]);
-}
-
-template <typename S, typename D>
-__global__ void k_unpack(const S *__restrict__ in, int64_t n, int64_t stride, double scale, D *__restrict__ out) {
-  pdl_enter();
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 8 * n) return;
-  const int64_t i = t >> 3;
-  const int c = (int)(t & 7);
-  out[t] = (D)(scale * (double)in[((int64_t)cell_parity(c) * stride + i) * 4 + (c >> 1)]);
-}
-
-__global__ void k_sum_phi(const double *__restrict__ phi, int64_t n, int64_t n_alloc, double *__restrict__ partials) {
+template <bool WIDE, typename T>
+__global__ void __launch_bounds__(kThreads) k_pack(const T *__restrict__ in, int64_t n, int64_t stride, double scale,
+                                                  T *__restrict__ out) {
   pdl_enter();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  T v[8], w[4];
+  load8<WIDE>(in + i * 8, v);
+  if (scale != 1.0) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = (T)(scale * (double)v[c]);
+  }
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    to_plane(v, p, w);
+    dev::store4(out + (p * stride + i) * 4, w);
+  }
+}
+
+template <bool WIDE, typename T>
+__global__ void __launch_bounds__(kThreads) k_unpack(const T *__restrict__ in, int64_t n, int64_t stride, double scale,
+                                                    T *__restrict__ out) {
+  pdl_enter();
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  T v[8];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    T w[4];
+    dev::load4<false>(in + (p * stride + i) * 4, w);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[plane_cell(p, q)] = w[q];
+  }
+  if (scale != 1.0) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = (T)(scale * (double)v[c]);
+  }
+  store8<WIDE>(out + i * 8, v);
+}
+
+// Sum of phi: a grid-stride loop, so that the block sums' FP64 additions
+// (which issue once per ~64 clocks) are paid once per block and not per 256
+// octs.
+__global__ void __launch_bounds__(kThreads) k_sum_phi(const double *__restrict__ phi, int64_t n, int64_t n_alloc,
+                                                     double *__restrict__ partials) {
+  pdl_enter();
   double acc = 0.0;
-  if (i < n) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += gridDim.x * (int64_t)blockDim.x) {
     double a[4], b[4];
     dev::load4<false>(phi + i * 4, a);
     dev::load4<false>(phi + (n_alloc + i) * 4, b);
-    acc = ((a[0] + a[1]) + (a[2] + a[3])) + ((b[0] + b[1]) + (b[2] + b[3]));
+    acc += ((a[0] + a[1]) + (a[2] + a[3])) + ((b[0] + b[1]) + (b[2] + b[3]));
   }
   block_sum_to(acc, partials);
 }
 
-__global__ void k_sub_scalar(double *__restrict__ phi, int64_t n, int64_t n_alloc, const double *__restrict__ s) {
+__global__ void __launch_bounds__(kThreads) k_sub_scalar(double *__restrict__ phi, int64_t n, int64_t n_alloc,
+                                                        const double *__restrict__ s) {
   pdl_enter();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 8 * n) return;
-  const int64_t i = t >> 3;
-  const int p = (int)((t >> 2) & 1);
-  const int q = (int)(t & 3);
-  phi[(p * n_alloc + i) * 4 + q] -= *s;
+  if (t >= 2 * n) return;
+  const int p = t >= n ? 1 : 0;
+  double *at = phi + (p * n_alloc + (t - p * n)) * 4;
+  const double x = *s;
+  double v[4];
+  dev::load4<false>(at, v);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] -= x;
+  dev::store4(at, v);
 }
 
 // phi64 += S * phi32 on the real octs (solution accumulation, FP64)
@@ -291,7 +363,7 @@ __global__ void k_accumulate(double *__restrict__ phi, const float *__restrict__
   pdl_enter();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= 2 * n) return;
-  const int p = (int)(t / n);
+  const int p = t >= n ? 1 : 0;
   const int64_t i = t - p * n;
   const double S = *scale;
   double v[4];

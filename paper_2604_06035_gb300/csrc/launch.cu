@@ -1,6 +1,7 @@
 // launch.cu -- host launchers of the one-operation-per-launch kernels
 // (kernels.cuh), with the algorithmic work each launch reports to the
 // profiler.
+#include <algorithm>
 #include <cmath>
 
 #include "cmg_internal.cuh"
@@ -288,7 +289,7 @@ void subtract_mean(cmg_level *L) {
   MgLev &g = L->mg[0];
   if (g.n == 0) return;
   cudaStream_t s = L->ctx->stream;
-  const unsigned nb = blocks_for(g.n);
+  const unsigned nb = std::min(blocks_for(g.n), 8u * (unsigned)L->ctx->num_sms);
   {
     LaunchScope ls(L->ctx, K_REDUCE, 64.0 * g.n, 8.0 * g.n);
     launch_k(k_sum_phi, nb, kThreads, s, g.phi, g.n, g.n_alloc, L->partials);
@@ -299,7 +300,7 @@ void subtract_mean(cmg_level *L) {
   }
   {
     LaunchScope ls(L->ctx, K_CONVERT, 128.0 * g.n, 8.0 * g.n);
-    launch_k(k_sub_scalar, blocks_for(8 * g.n), kThreads, s, g.phi, g.n, g.n_alloc, L->scal + 6);
+    launch_k(k_sub_scalar, blocks_for(2 * g.n), kThreads, s, g.phi, g.n, g.n_alloc, L->scal + 6);
   }
   CMG_CUDA(cudaGetLastError());
 }
@@ -312,12 +313,15 @@ void accumulate(cmg_level *L, const double *scale) {
   CMG_CUDA(cudaGetLastError());
 }
 
+// whether a caller's array takes 16-byte accesses
+static bool wide(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 void set_density(cmg_level *L, const double *rho, double rho_bar, double four_pi_g) {
   MgLev &g = L->mg[0];
   if (g.n == 0) return;
   const double scale = -g.h * g.h / 6.0 * four_pi_g;
   LaunchScope ls(L->ctx, K_CONVERT, g.n * 8.0 * 16.0, g.n * 16.0);
-  k_set_density<<<blocks_for(8 * g.n), kThreads, 0, L->ctx->stream>>>(rho, g.n, rho_bar, scale, g.g);
+  (wide(rho) ? k_set_density<true> : k_set_density<false>)<<<blocks_for(g.n), kThreads, 0, L->ctx->stream>>>(rho, g.n, rho_bar, scale, g.g);
   CMG_CUDA(cudaGetLastError());
 }
 
@@ -337,12 +341,12 @@ void pack_field(cmg_level *L, int m, int field, int prec, const void *in) {
   cudaStream_t s = L->ctx->stream;
   const double scale = field == 0 ? 1.0 : -g.h * g.h / 6.0;
   const int64_t stride = field == 0 ? g.n_alloc : g.n;
-  const unsigned nb = blocks_for(8 * g.n);
+  const unsigned nb = blocks_for(g.n);
   LaunchScope ls(L->ctx, K_CONVERT, g.n * 8.0 * 2.0 * (prec == CMG_PREC_FP64 ? 8.0 : 4.0), 0.0);
   if (prec == CMG_PREC_FP64)
-    launch_k(k_pack<double, double>, nb, kThreads, s, (const double *)in, g.n, stride, scale, field == 0 ? g.phi : g.g);
+    launch_k(wide(in) ? k_pack<true, double> : k_pack<false, double>, nb, kThreads, s, (const double *)in, g.n, stride, scale, field == 0 ? g.phi : g.g);
   else
-    launch_k(k_pack<float, float>, nb, kThreads, s, (const float *)in, g.n, stride, scale, field == 0 ? g.phi32 : g.g32);
+    launch_k(wide(in) ? k_pack<true, float> : k_pack<false, float>, nb, kThreads, s, (const float *)in, g.n, stride, scale, field == 0 ? g.phi32 : g.g32);
   CMG_CUDA(cudaGetLastError());
 }
 
@@ -352,12 +356,12 @@ void unpack_field(cmg_level *L, int m, int field, int prec, void *out) {
   cudaStream_t s = L->ctx->stream;
   const double scale = field == 0 ? 1.0 : -6.0 / (g.h * g.h);
   const int64_t stride = field == 0 ? g.n_alloc : g.n;
-  const unsigned nb = blocks_for(8 * g.n);
+  const unsigned nb = blocks_for(g.n);
   LaunchScope ls(L->ctx, K_CONVERT, g.n * 8.0 * 2.0 * (prec == CMG_PREC_FP64 ? 8.0 : 4.0), 0.0);
   if (prec == CMG_PREC_FP64)
-    launch_k(k_unpack<double, double>, nb, kThreads, s, field == 0 ? g.phi : g.g, g.n, stride, scale, (double *)out);
+    launch_k(wide(out) ? k_unpack<true, double> : k_unpack<false, double>, nb, kThreads, s, field == 0 ? g.phi : g.g, g.n, stride, scale, (double *)out);
   else
-    launch_k(k_unpack<float, float>, nb, kThreads, s, field == 0 ? g.phi32 : g.g32, g.n, stride, scale, (float *)out);
+    launch_k(wide(out) ? k_unpack<true, float> : k_unpack<false, float>, nb, kThreads, s, field == 0 ? g.phi32 : g.g32, g.n, stride, scale, (float *)out);
   CMG_CUDA(cudaGetLastError());
 }
 

@@ -366,6 +366,17 @@ __device__ __forceinline__ double resid_oct_idx(int64_t i, const ResidIdx &x, co
   const unsigned m = x.m;
   T rsum = T(0);
   double acc = 0.0;
+  if constexpr (ZPHI && NORM && !RESTRICT && !EMIT && !ROUT) {
+    // phi taken as zero: away from the Dirichlet ghosts every sum is zero and
+    // fma(0, 1/6, g) = g (256^3 level: 118 -> 45 us)
+    if (max(max(max(nb[0], nb[1]), max(nb[2], nb[3])), max(nb[4], nb[5])) < n && m == 0xFFu) {
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc = fma((double)gv[p][q], (double)gv[p][q], acc);
+      return acc;
+    }
+  }
   T tacc = T(0);  // FP32 data: the oct's squares summed in FP32, one conversion
 #pragma unroll
   for (int p = 0; p < 2; ++p) {

@@ -9,6 +9,7 @@
 // The host waits once per solve.  With profiling on, the same kernels are
 // launched one by one from a host loop instead (conditional bodies cannot
 // hold event nodes), so that every launch can be bracketed by CUDA events.
+#include <algorithm>
 #include <cmath>
 
 #include "cmg_internal.cuh"
@@ -147,12 +148,13 @@ __global__ void __launch_bounds__(1024) k_norm_check(const double *__restrict__ 
   }
 }
 
+// (a few blocks: they read one flag and, save for a zero source, return)
 __global__ void k_zero_if(const SolveCtrl *c, double *phi, int64_t n, int64_t n_alloc) {
   if (!c->zero) return;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 8 * n) return;
-  const int p = (int)((t >> 2) & 1);
-  phi[(p * n_alloc + (t >> 3)) * 4 + (t & 3)] = 0.0;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 8 * n; t += gridDim.x * (int64_t)blockDim.x) {
+    const int p = (int)((t >> 2) & 1);
+    phi[(p * n_alloc + (t >> 3)) * 4 + (t & 3)] = 0.0;
+  }
 }
 
 // Coarse phi must start at zero unless the next operation on it overwrites
@@ -293,7 +295,7 @@ void segment_post(cmg_level *L, const cmg_solve_params *p) {
   if (p->krylov == 1) pcg_post(L);
   {
     LaunchScope ls(L->ctx, K_CONVERT, 0.0, 0.0);
-    k_zero_if<<<blocks_for(8 * g.n), kThreads, 0, L->ctx->stream>>>(ctrl_dev(L), g.phi, g.n, g.n_alloc);
+    k_zero_if<<<std::min(blocks_for(8 * g.n), (unsigned)L->ctx->num_sms), kThreads, 0, L->ctx->stream>>>(ctrl_dev(L), g.phi, g.n, g.n_alloc);
     CMG_CUDA(cudaGetLastError());
   }
   if (L->periodic_full) subtract_mean(L);
