@@ -139,16 +139,16 @@ __global__ void __launch_bounds__(kThreads) k_resid(const int32_t *__restrict__ 
     if (i < n) x = dev::resid_idx<RESTRICT>(i, nbr, active, n, father);
     pdl_enter();
     if (i < n) {
-      const double inv_s = EMIT ? 1.0 / *emit_scale : 0.0;
-      acc = dev::resid_oct_idx<T, NORM, RESTRICT, EMIT, ROUT, ZPHI, false, C1Z>(i, x, phi, g, n, n_alloc, cg, cphi, cn,
+      const double inv_s = EMIT ? dev::inv_scale(*emit_scale) : 0.0;
+      acc = dev::resid_oct_idx<T, NORM, RESTRICT, EMIT, ROUT, ZPHI, false, C1Z, C1Z>(i, x, phi, g, n, n_alloc, cg, cphi, cn,
                                                                            cn_alloc, zero_cphi, g32, inv_s, rout,
                                                                            rscale);
     }
   } else {
     pdl_enter();
     if (i < n) {
-      const double inv_s = EMIT ? 1.0 / *emit_scale : 0.0;
-      acc = dev::resid_oct<T, NORM, RESTRICT, EMIT, ROUT, ZPHI, false, C1Z>(i, nbr, phi, g, active, n, n_alloc, father,
+      const double inv_s = EMIT ? dev::inv_scale(*emit_scale) : 0.0;
+      acc = dev::resid_oct<T, NORM, RESTRICT, EMIT, ROUT, ZPHI, false, C1Z, C1Z>(i, nbr, phi, g, active, n, n_alloc, father,
                                                                        cg, cphi, cn, cn_alloc, zero_cphi, g32, inv_s,
                                                                        rout, rscale);
     }
@@ -371,7 +371,7 @@ __global__ void k_accumulate(double *__restrict__ phi, const float *__restrict__
   dev::load4<false>(phi + (p * n_alloc + i) * 4, v);
   dev::load4<false>(e + (p * n_alloc + i) * 4, w);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) v[q] = fma(S, (double)w[q], v[q]);
+  for (int q = 0; q < 4; ++q) v[q] = fma(S, dev::widen(w[q]), v[q]);
   dev::store4(phi + (p * n_alloc + i) * 4, v);
 }
 

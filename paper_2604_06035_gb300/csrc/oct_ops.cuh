@@ -221,46 +221,52 @@ __device__ __forceinline__ SweepIdx sweep_idx(int64_t i, const int32_t *__restri
   return x;
 }
 
-template <typename T, int P, bool ZERO, bool MASK, bool CG>
-__device__ __forceinline__ void sweep_oct_idx(int64_t i, const SweepIdx &x, const T *src, T *dst, const T *g) {
-  T gv[4], out[4];
-  load4<CG>(g + i * 4, gv);
-  if (ZERO) {
+// The values a pass reads for an oct, apart from the arithmetic on them, so
+// that a loop over octs can have the next oct's in flight.
+template <typename T>
+struct SweepVals {
+  T g[4], own[4], nb[6][4];
+};
+template <typename T, bool ZERO, bool CG>
+__device__ __forceinline__ void sweep_load(int64_t i, const SweepIdx &x, const T *src, const T *g, SweepVals<T> &v) {
+  load4<CG>(g + i * 4, v.g);
+  if (ZERO) return;
+  load4<CG>(src + i * 4, v.own);
+  // whole neighbour octs, two of their values used each: fewer, wider loads
+  // than one per value (256^3 + 3-level chains: FP32 passes 16.95 -> 16.35
+  // ms per step, FP64 ones 26.96 -> 26.52)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out[q] = gv[q];
-  } else {
-    T own[4];
-    load4<CG>(src + i * 4, own);
-    const int32_t *nb = x.nb;
-    const T inv6 = T(1) / T(6);
-    // whole neighbour octs, two of their values used each: fewer, wider loads
-    // than one per value (256^3 + 3-level chains: FP32 passes 16.95 -> 16.35
-    // ms per step, FP64 ones 26.96 -> 26.52)
-    T nv[6][4];
-    if (!CG) {
+  for (int d = 0; d < 6; ++d) {
+    if (CG) load4<CG>(src + (int64_t)x.nb[d] * 4, v.nb[d]);
+    else load_oct(src + (int64_t)x.nb[d] * 4, v.nb[d]);
+  }
+}
+template <typename T, int P, bool ZERO, bool MASK>
+__device__ __forceinline__ void sweep_finish(int64_t i, const SweepIdx &x, const SweepVals<T> &w, T *dst) {
+  T out[4];
 #pragma unroll
-      for (int d = 0; d < 6; ++d) load_oct(src + (int64_t)nb[d] * 4, nv[d]);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = plane_cell(P, q);
+  for (int q = 0; q < 4; ++q) {
+    const int c = plane_cell(P, q);
+    out[q] = w.g[q];
+    if (!ZERO) {
       T v[6];
 #pragma unroll
       for (int d = 0; d < 6; ++d) {
         const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
-        if (((c >> a) & 1) != side) v[d] = own[c2 >> 1];
-        else if (!CG) v[d] = nv[d][c2 >> 1];
-        else v[d] = ld1<CG>(src + (int64_t)nb[d] * 4 + (c2 >> 1));
+        v[d] = ((c >> a) & 1) != side ? w.own[c2 >> 1] : w.nb[d][c2 >> 1];
       }
-      out[q] = fma_t(nbsum6(v), inv6, gv[q]);
+      out[q] = fma_t(nbsum6(v), T(1) / T(6), out[q]);
     }
-  }
-  if (MASK) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (!((x.m >> plane_cell(P, q)) & 1)) out[q] = T(0);
+    if (MASK && !((x.m >> c) & 1)) out[q] = T(0);
   }
   store4(dst + i * 4, out);
+}
+
+template <typename T, int P, bool ZERO, bool MASK, bool CG>
+__device__ __forceinline__ void sweep_oct_idx(int64_t i, const SweepIdx &x, const T *src, T *dst, const T *g) {
+  SweepVals<T> v;
+  sweep_load<T, ZERO, CG>(i, x, src, g, v);
+  sweep_finish<T, P, ZERO, MASK>(i, x, v, dst);
 }
 
 template <typename T, int P, bool ZERO, bool MASK, bool CG>
@@ -319,6 +325,20 @@ __device__ __forceinline__ float f32_scaled(double x, double s) {
   const uint32_t m = (uint32_t)((mant + 0x0FFFFFFFull + ((mant >> 29) & 1ull)) >> 29);
   return __uint_as_float((((uint32_t)fe << 23) + m) | ((uint32_t)(xb >> 32) & 0x80000000u));
 }
+// (double)x in integer operations (the conversion issues on the FP64 pipe).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), m = b & 0x7FFFFFFFu;
+  if (m - 0x00800000u >= 0x7F000000u && m != 0) return (double)x;  // subnormal, infinite, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(b << 29));
+}
+// 1 / s: exact and without the FP64 pipe's ten-odd instructions for a normal
+// power of two.
+__device__ __forceinline__ double inv_scale(double s) {
+  const int hi = __double2hiint(s);
+  if ((hi & 0x800FFFFF) == 0 && __double2loint(s) == 0 && hi >= 0x00100000 && hi <= 0x7FD00000)
+    return __hiloint2double(0x7FE00000 - hi, 0);
+  return 1.0 / s;
+}
 struct ResidIdx {
   int32_t nb[6];
   unsigned m;
@@ -346,7 +366,14 @@ __device__ __forceinline__ ResidIdx resid_idx(int64_t i, const int32_t *__restri
 // +0 terms (acc >= +0 throughout), the restriction sum would gain +0 four
 // times, which leaves it unchanged (it is never -0), and EMIT / ROUT write
 // what dv = +0 gives.
-template <typename T, bool NORM, bool RESTRICT, bool EMIT, bool ROUT, bool ZPHI, bool CG, bool C1Z = false>
+//
+// WIDE: the neighbours' planes in one access each (as in sweep_load) instead
+// of value by value.  For the colour-0 residuals alone it is faster (batch of
+// 512 patches: restriction 570 -> 447 us, norm 631 -> 519 us), for both
+// colours' its registers cost the one-launch kernels occupancy (256^3 mixed
+// chain 23.9 -> 24.3 ms).
+template <typename T, bool NORM, bool RESTRICT, bool EMIT, bool ROUT, bool ZPHI, bool CG, bool C1Z = false,
+          bool WIDE = false>
 __device__ __forceinline__ double resid_oct_idx(int64_t i, const ResidIdx &x, const T *phi, const T *g, int64_t n,
                                                 int64_t n_alloc, T *cg, T *cphi, int64_t cn, int64_t cn_alloc,
                                                 int zero_cphi, float *g32, double inv_s, double *rout,
@@ -390,6 +417,16 @@ __device__ __forceinline__ double resid_oct_idx(int64_t i, const ResidIdx &x, co
       }
       continue;
     }
+    // the neighbours' other planes, whole (as in sweep_load)
+    T nv[6][4];
+    if (WIDE && !ZPHI) {
+#pragma unroll
+      for (int d = 0; d < 6; ++d) {
+        const T *at = phi + ((1 - p) * n_alloc + (int64_t)nb[d]) * 4;
+        if (CG) load4<CG>(at, nv[d]);
+        else load_oct(at, nv[d]);
+      }
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int c = plane_cell(p, q);
@@ -399,6 +436,8 @@ __device__ __forceinline__ double resid_oct_idx(int64_t i, const ResidIdx &x, co
         const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
         if (((c >> a) & 1) != side) {
           v[d] = pl[1 - p][c2 >> 1];
+        } else if (WIDE && !ZPHI) {
+          v[d] = nv[d][c2 >> 1];
         } else {
           const int64_t o = nb[d];
           v[d] = (ZPHI && o < n) ? T(0) : ld1<CG>(phi + ((1 - p) * n_alloc + o) * 4 + (c2 >> 1));
@@ -430,13 +469,14 @@ __device__ __forceinline__ double resid_oct_idx(int64_t i, const ResidIdx &x, co
   return acc;
 }
 
-template <typename T, bool NORM, bool RESTRICT, bool EMIT, bool ROUT, bool ZPHI, bool CG, bool C1Z = false>
+template <typename T, bool NORM, bool RESTRICT, bool EMIT, bool ROUT, bool ZPHI, bool CG, bool C1Z = false,
+          bool WIDE = false>
 __device__ __forceinline__ double resid_oct(int64_t i, const int32_t *__restrict__ nbr, const T *phi, const T *g,
                                             const uint8_t *__restrict__ active, int64_t n, int64_t n_alloc,
                                             const int32_t *__restrict__ father, T *cg, T *cphi, int64_t cn,
                                             int64_t cn_alloc, int zero_cphi, float *g32, double inv_s,
                                             double *rout, double rscale) {
-  return resid_oct_idx<T, NORM, RESTRICT, EMIT, ROUT, ZPHI, CG, C1Z>(i, resid_idx<RESTRICT>(i, nbr, active, n, father),
+  return resid_oct_idx<T, NORM, RESTRICT, EMIT, ROUT, ZPHI, CG, C1Z, WIDE>(i, resid_idx<RESTRICT>(i, nbr, active, n, father),
                                                                 phi, g, n, n_alloc, cg, cphi, cn, cn_alloc,
                                                                 zero_cphi, g32, inv_s, rout, rscale);
 }
