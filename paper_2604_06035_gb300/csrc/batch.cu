@@ -43,6 +43,10 @@ struct BatchPlan {
   long long spin_budget;
   BLevel lv[kBMaxLevels];
   const int32_t *pid;  // patch of each top-level oct
+  // levels split .. depth - 1 are worked on block by block (depth: none): block
+  // b's patches hold the octs first[m (gridDim.x + 1) + b] .. of level m
+  int split;
+  const int32_t *first;
   // Dirichlet ghosts of the top level
   int64_t n_ghost;
   const uint64_t *gkeys;
@@ -73,6 +77,67 @@ __device__ bool grid_sync(const BatchPlan &P) {
   return true;
 }
 
+// The octs of a level (or cells, k per oct) that a thread handles: a, a + s, ...
+// below e.
+struct Octs {
+  int64_t a, e, s;
+};
+
+// Who works on a level and what separates dependent operations.
+//
+// All: the whole grid on the whole level, grid barriers.  The grid walks a
+// level as one window, which keeps the neighbours' values in L2 (one
+// contiguous chunk per block instead, 304 windows: 512-patch FP64 solve 155 ->
+// 243 ms).  A level that the threads take in one round is dealt out warp by
+// warp, so that every SM gets its share.
+struct All {
+  const BatchPlan &P;
+  __device__ __forceinline__ Octs units(int m, int k) const {
+    const int64_t e = k * P.lv[m].n, s = (int64_t)gridDim.x * blockDim.x;
+    if (e <= s) return {((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31), e, s};
+    return {(int64_t)blockIdx.x * blockDim.x + threadIdx.x, e, s};
+  }
+  static constexpr bool kCells = false;
+  __device__ __forceinline__ bool per_cell(int) const { return false; }
+  __device__ __forceinline__ bool sync() const { return grid_sync(P); }
+};
+// Own: each block the octs of its own patches, block barriers.  On the coarse
+// levels, whose octs take a round or two of a block's threads, a grid barrier
+// and the first touch of other SMs' data are most of an operation's 2 to 3.5
+// us.
+struct Own {
+  const BatchPlan &P;
+  __device__ __forceinline__ int64_t at(int m, int k) const {
+    return __ldg(P.first + (int64_t)m * (gridDim.x + 1) + blockIdx.x + k);
+  }
+  __device__ __forceinline__ Octs units(int m, int k) const {
+    return {k * at(m, 0) + threadIdx.x, k * at(m, 1), (int64_t)blockDim.x};
+  }
+  static constexpr bool kCells = true;
+  __device__ __forceinline__ bool per_cell(int m) const { return 4 * (at(m, 1) - at(m, 0)) <= (int64_t)blockDim.x; }
+  __device__ __forceinline__ bool sync() const {
+    __syncthreads();
+    return true;
+  }
+};
+
+// Calls body(i, x) for every STEP-th oct of the thread, x = idx(i) its index
+// data, read while the oct before it is worked on.
+template <int STEP, class Idx, class Body>
+__device__ __forceinline__ void for_octs(const Octs o, Idx idx, Body body) {
+  int64_t i = o.a;
+  if (i >= o.e) return;
+  auto x = idx(i);
+  for (;;) {
+    const int64_t j = i + STEP * o.s;
+    auto y = idx(j < o.e ? j : i);
+    body(i, x);
+    if (j >= o.e) return;
+    i = j;
+    x = y;
+  }
+}
+
 // Sum v over the lanes of the warp that share patch p (p < 0: no value).
 __device__ __forceinline__ void patch_add(double *arr, int p, double v) {
   const int lane = threadIdx.x & 31;
@@ -84,6 +149,45 @@ __device__ __forceinline__ void patch_add(double *arr, int p, double v) {
   } else if (p >= 0) {
     atomicAdd(arr + p, v);
   }
+}
+
+// patch_add over a loop: while a warp stays within one patch each lane keeps
+// its own sum (one FP64 addition instead of a warp reduction per 32 octs).
+// Every lane of the warp makes the same calls.
+struct PatchSum {
+  double *arr;
+  int cur = -1;  // the warp's patch
+  double acc = 0.0;
+  __device__ __forceinline__ void add(int p, double v) {
+    const int p0 = __shfl_sync(0xffffffffu, p, 0);
+    const bool same = __all_sync(0xffffffffu, p == p0 || p < 0);
+    if (same && p0 == cur) {
+      acc += v;
+      return;
+    }
+    flush();
+    if (same) {
+      cur = p0;
+      acc = v;
+    } else if (p >= 0) {
+      atomicAdd(arr + p, v);
+    }
+  }
+  __device__ __forceinline__ void flush() {
+    if (cur >= 0) patch_add(arr, cur, acc);
+    cur = -1;
+    acc = 0.0;
+  }
+};
+
+// The FP32 right-hand sides' scale for a norm: the power of two of its binade
+// (products with it are exact), itself if infinite, else 1.
+__device__ __forceinline__ double pow2_scale(double v) {
+  if (!(v > 0.0)) return 1.0;
+  if (v == INFINITY) return v;
+  int e;
+  (void)frexp(v, &e);
+  return ldexp(1.0, e - 1);
 }
 
 template <typename T>
@@ -107,97 +211,194 @@ __device__ __forceinline__ T *g_t(const BLevel &L) {
 #endif
 constexpr bool kCG = CMG_BATCH_CG != 0;
 
-template <typename T>
-__device__ void colour_pass(const BLevel &L, int P, bool zero, int64_t tid, int64_t nthr, T *phi, const T *g) {
+// One colour pass.  FP32: two octs at a time, the loads of both in flight
+// together (FP64 values would take the registers).  A block's own FP64 octs
+// run one thread per cell where that is one round (the FP64 instructions would
+// leave most lanes idle and follow one another in one); the same for
+// restriction and prolongation below.
+template <typename T, int P, bool ZERO, bool MASK, class W>
+__device__ __noinline__ void pass(const W on, int m, T *phi, const T *g) {
+  const BLevel L = on.P.lv[m];  // by value: the loops' loads would have it read again each time
   const int64_t st = L.n_alloc * 4;
-  for (int64_t i = tid; i < L.n; i += nthr) {
-    if (P == 0) {
-      if (zero) {
-        if (L.all_active) dev::sweep_oct<T, 0, true, false, kCG>(i, L.nbr, phi + st, phi, g, L.active, L.n);
-        else dev::sweep_oct<T, 0, true, true, kCG>(i, L.nbr, phi + st, phi, g, L.active, L.n);
-      } else {
-        if (L.all_active) dev::sweep_oct<T, 0, false, false, kCG>(i, L.nbr, phi + st, phi, g, L.active, L.n);
-        else dev::sweep_oct<T, 0, false, true, kCG>(i, L.nbr, phi + st, phi, g, L.active, L.n);
-      }
-    } else {
-      if (L.all_active) dev::sweep_oct<T, 1, false, false, kCG>(i, L.nbr, phi, phi + st, g + L.n * 4, L.active, L.n);
-      else dev::sweep_oct<T, 1, false, true, kCG>(i, L.nbr, phi, phi + st, g + L.n * 4, L.active, L.n);
+  const T *src = P == 0 ? phi + st : phi, *gp = P == 0 ? g : g + L.n * 4;
+  T *dst = P == 0 ? phi : phi + st;
+  if constexpr (sizeof(T) == 8) {
+    if (W::kCells && on.per_cell(m)) {
+      const Octs o = on.units(m, 4);
+      for (int64_t u = o.a; u < o.e; u += o.s)
+        dev::sweep_cell<T, P, ZERO, MASK, kCG>(u >> 2, (int)(u & 3), L.nbr, src, dst, gp, L.active, L.n);
+      return;
     }
+    for_octs<1>(on.units(m, 1), [&](int64_t i) { return dev::sweep_idx<ZERO, MASK>(i, L.nbr, L.active, L.n); },
+                [&](int64_t i, const dev::SweepIdx &x) { dev::sweep_oct_idx<T, P, ZERO, MASK, kCG>(i, x, src, dst, gp); });
+  } else {
+    const Octs o = on.units(m, 1);
+    struct Two {
+      dev::SweepIdx x[2];
+    };
+    for_octs<2>(o,
+                [&](int64_t i) {
+                  return Two{{dev::sweep_idx<ZERO, MASK>(i, L.nbr, L.active, L.n),
+                              dev::sweep_idx<ZERO, MASK>(i + o.s < o.e ? i + o.s : i, L.nbr, L.active, L.n)}};
+                },
+                [&](int64_t i, const Two &t) {
+                  const int64_t j = i + o.s < o.e ? i + o.s : i;  // twice the same at the end: the same values
+                  dev::SweepVals<T> v, w;
+                  dev::sweep_load<T, ZERO, kCG>(i, t.x[0], src, gp, v);
+                  dev::sweep_load<T, ZERO, kCG>(j, t.x[1], src, gp, w);
+                  dev::sweep_finish<T, P, ZERO, MASK>(i, t.x[0], v, dst);
+                  dev::sweep_finish<T, P, ZERO, MASK>(j, t.x[1], w, dst);
+                });
+  }
+}
+template <typename T, class W>
+__device__ void colour_pass(const W &on, int m, int P, bool zero, T *phi, const T *g) {
+  if (on.P.lv[m].all_active) {
+    if (P == 1) pass<T, 1, false, false>(on, m, phi, g);
+    else if (zero) pass<T, 0, true, false>(on, m, phi, g);
+    else pass<T, 0, false, false>(on, m, phi, g);
+  } else {
+    if (P == 1) pass<T, 1, false, true>(on, m, phi, g);
+    else if (zero) pass<T, 0, true, true>(on, m, phi, g);
+    else pass<T, 0, false, true>(on, m, phi, g);
   }
 }
 
-template <typename T>
-__device__ bool sweeps(const BatchPlan &Pl, const BLevel &L, int n_sweeps, bool zero_first, int64_t tid,
-                       int64_t nthr, T *phi, const T *g) {
+template <typename T, class W>
+__device__ bool sweeps(const W &on, int m, int n_sweeps, bool zero_first) {
+  const BLevel &L = on.P.lv[m];
   for (int k = 0; k < n_sweeps; ++k) {
-    colour_pass<T>(L, 0, zero_first && k == 0, tid, nthr, phi, g);
-    if (!grid_sync(Pl)) return false;
-    colour_pass<T>(L, 1, false, tid, nthr, phi, g);
-    if (!grid_sync(Pl)) return false;
+    colour_pass<T>(on, m, 0, zero_first && k == 0, phi_t<T>(L), g_t<T>(L));
+    if (!on.sync()) return false;
+    colour_pass<T>(on, m, 1, false, phi_t<T>(L), g_t<T>(L));
+    if (!on.sync()) return false;
   }
   return true;
+}
+
+// Residuals of level m restricted to m + 1; C1Z: see resid_oct_idx.
+template <typename T, bool C1Z, class W>
+__device__ __noinline__ void restrict_residual(const W on, int m, int zero_coarse) {
+  const BLevel L = on.P.lv[m], C = on.P.lv[m + 1];
+  const uint8_t *act = L.all_active ? nullptr : L.active;
+  if constexpr (sizeof(T) == 8 && W::kCells) {
+    if (on.per_cell(m)) {  // the 8 lanes of an oct exchange values: whole warps
+      const Octs o = on.units(m, 8);
+      const int lane = threadIdx.x & 31;
+      for (int64_t b = o.a - lane; b < o.e; b += o.s)
+        dev::resid_restrict_cell<T, kCG>(b + lane < o.e, (b + lane) >> 3, L.nbr, L.phi, L.g, act, L.n, L.n_alloc,
+                                         L.father, C.g, C.phi, C.n, C.n_alloc, zero_coarse);
+      return;
+    }
+  }
+  for_octs<1>(on.units(m, 1), [&](int64_t i) { return dev::resid_idx<true>(i, L.nbr, act, L.n, L.father); },
+              [&](int64_t i, const dev::ResidIdx &x) {
+                dev::resid_oct_idx<T, false, true, false, false, false, kCG, C1Z, true>(
+                    i, x, phi_t<T>(L), g_t<T>(L), L.n, L.n_alloc, g_t<T>(C), phi_t<T>(C), C.n, C.n_alloc, zero_coarse,
+                    nullptr, 0.0, nullptr, 0.0);
+              });
+}
+
+// Prolongation of m + 1 added to m.  C0D: a colour-0 pass comes next and
+// overwrites the colour-0 corrections unread.
+template <typename T, bool MASK, bool C0D, class W>
+__device__ __noinline__ void prolong(const W on, int m) {
+  const BLevel L = on.P.lv[m], C = on.P.lv[m + 1];
+  if constexpr (sizeof(T) == 8 && W::kCells) {
+    if (on.per_cell(m)) {
+      const Octs o = on.units(m, C0D ? 4 : 8);
+      for (int64_t u = o.a; u < o.e; u += o.s)
+        dev::prolong_cell<T, MASK, kCG>(C0D ? u >> 2 : u >> 3, C0D ? plane_cell(1, (int)(u & 3)) : (int)(u & 7), L.keys,
+                                        L.blk, L.n, L.n_alloc, L.phi, L.active, C.phi, C.n_alloc);
+      return;
+    }
+  }
+  for_octs<1>(on.units(m, 1), [&](int64_t i) { return dev::prolong_idx<MASK>(i, L.keys, L.blk, L.n, L.active); },
+              [&](int64_t i, const dev::ProlongIdx &x) {
+                dev::prolong_oct_idx<T, MASK, kCG, C0D>(i, x, L.n_alloc, phi_t<T>(L), phi_t<T>(C), C.n_alloc);
+              });
+}
+
+// Down leg over levels [from, to): pre-smoothing of m, its residual restricted
+// to m + 1.
+template <typename T, class W>
+__device__ bool descend(const W &on, int from, int to, bool zero_top) {
+  const BatchPlan &P = on.P;
+  for (int m = from; m < to; ++m) {
+    if (!sweeps<T>(on, m, P.n_pre, m > 0 || zero_top)) return false;
+    const int zc = (m + 2 < P.depth) ? (P.n_pre == 0) : (P.n_pre + P.n_post == 0);
+    // after pre-smoothing (n_pre >= 1) the colour-1 residuals are exactly 0
+    if (P.n_pre >= 1) restrict_residual<T, true>(on, m, zc);
+    else restrict_residual<T, false>(on, m, zc);
+    if (!on.sync()) return false;
+  }
+  return true;
+}
+
+// The coarsest level: n_pre + n_post sweeps, in FP64 (on FP64 copies).
+template <typename T, class W>
+__device__ bool coarsest(const W &on) {
+  const BatchPlan &P = on.P;
+  const int last = P.depth - 1, nsw = P.n_pre + P.n_post;
+  const BLevel &L = P.lv[last];
+  if constexpr (sizeof(T) == 4) {
+    const Octs o = on.units(last, 4);
+    for (int p = 0; p < 2; ++p)
+      for (int64_t t = o.a; t < o.e; t += o.s) L.g[p * 4 * L.n + t] = (double)__ldcg(L.g32 + p * 4 * L.n + t);
+    if (!on.sync()) return false;
+    if (!sweeps<double>(on, last, nsw, last > 0)) return false;
+    // (the octs beyond the real ones are zero in both precisions)
+    for (int p = 0; p < 2; ++p)
+      for (int64_t t = o.a; t < o.e; t += o.s)
+        L.phi32[p * 4 * L.n_alloc + t] = (float)__ldcg(L.phi + p * 4 * L.n_alloc + t);
+    return on.sync();
+  } else {
+    return sweeps<T>(on, last, nsw, last > 0);
+  }
+}
+
+// Up leg from level `from` down to `to`: prolongation, post-smoothing.
+template <typename T, class W>
+__device__ bool ascend(const W &on, int from, int to) {
+  const BatchPlan &P = on.P;
+  for (int m = from; m >= to; --m) {
+    if (P.n_post >= 1) {
+      if (P.lv[m].all_active) prolong<T, false, true>(on, m);
+      else prolong<T, true, true>(on, m);
+    } else {
+      if (P.lv[m].all_active) prolong<T, false, false>(on, m);
+      else prolong<T, true, false>(on, m);
+    }
+    if (!on.sync()) return false;
+    if (!sweeps<T>(on, m, P.n_post, false)) return false;
+  }
+  return true;
+}
+
+// The V-cycle on the levels that the blocks work on by themselves (a call of
+// its own: inlined, its registers would be the other levels' spills).
+template <typename T>
+__device__ void own_levels(const BatchPlan &P, bool zero_top) {
+  const Own own{P};
+  descend<T>(own, P.split, P.depth - 1, zero_top);
+  coarsest<T>(own);
+  ascend<T>(own, P.depth - 2, P.split);
 }
 
 // One V-cycle over every MG level of the batch; T = double works on phi/g
 // (solution at the top, with ghosts), T = float on the FP32 correction.
 template <typename T>
-__device__ bool vcycle(const BatchPlan &P, bool zero_top, int64_t tid, int64_t nthr) {
-  const int last = P.depth - 1;
-  const int nsw = P.n_pre + P.n_post;  // coarsest solve = n_pre + n_post sweeps
-  for (int m = 0; m < last; ++m) {
-    const BLevel &L = P.lv[m];
-    const BLevel &C = P.lv[m + 1];
-    if (!sweeps<T>(P, L, P.n_pre, m > 0 || zero_top, tid, nthr, phi_t<T>(L), g_t<T>(L))) return false;
-    const int zc = (m + 1 < last) ? (P.n_pre == 0) : (nsw == 0);
-    // after pre-smoothing (n_pre >= 1) the colour-1 residuals are exactly 0
-    if (P.n_pre >= 1) {
-      for (int64_t i = tid; i < L.n; i += nthr)
-        dev::resid_oct<T, false, true, false, false, false, kCG, true>(
-            i, L.nbr, phi_t<T>(L), g_t<T>(L), L.all_active ? nullptr : L.active, L.n, L.n_alloc, L.father,
-            g_t<T>(C), phi_t<T>(C), C.n, C.n_alloc, zc, nullptr, 0.0, nullptr, 0.0);
-    } else {
-      for (int64_t i = tid; i < L.n; i += nthr)
-        dev::resid_oct<T, false, true, false, false, false, kCG>(
-            i, L.nbr, phi_t<T>(L), g_t<T>(L), L.all_active ? nullptr : L.active, L.n, L.n_alloc, L.father,
-            g_t<T>(C), phi_t<T>(C), C.n, C.n_alloc, zc, nullptr, 0.0, nullptr, 0.0);
-    }
-    if (!grid_sync(P)) return false;
+__device__ bool vcycle(const BatchPlan &P, bool zero_top) {
+  const All all{P};
+  const int last = P.depth - 1, mid = P.split < last ? P.split : last;
+  if (!descend<T>(all, 0, mid, zero_top)) return false;
+  if (P.split < P.depth) {
+    own_levels<T>(P, zero_top);
+    if (!all.sync()) return false;
+  } else if (!coarsest<T>(all)) {
+    return false;
   }
-  {
-    const BLevel &L = P.lv[last];
-    if (sizeof(T) == 4) {
-      // the coarsest level is solved in FP64 on FP64 copies
-      for (int64_t t = tid; t < 8 * L.n; t += nthr) L.g[t] = (double)__ldcg(L.g32 + t);
-      if (!grid_sync(P)) return false;
-      if (!sweeps<double>(P, L, nsw, last > 0, tid, nthr, L.phi, L.g)) return false;
-      for (int64_t t = tid; t < 8 * L.n_alloc; t += nthr) L.phi32[t] = (float)__ldcg(L.phi + t);
-      if (!grid_sync(P)) return false;
-    } else {
-      if (!sweeps<T>(P, L, nsw, last > 0, tid, nthr, phi_t<T>(L), g_t<T>(L))) return false;
-    }
-  }
-  for (int m = last - 1; m >= 0; --m) {
-    const BLevel &L = P.lv[m];
-    const BLevel &C = P.lv[m + 1];
-    // with post-smoothing, the colour-0 corrections are overwritten unread
-    for (int64_t i = tid; i < L.n; i += nthr) {
-      if (L.all_active && P.n_post >= 1)
-        dev::prolong_oct<T, false, kCG, true>(i, L.keys, L.blk, L.n, L.n_alloc, phi_t<T>(L), L.active, phi_t<T>(C),
-                                               C.n_alloc);
-      else if (L.all_active)
-        dev::prolong_oct<T, false, kCG>(i, L.keys, L.blk, L.n, L.n_alloc, phi_t<T>(L), L.active, phi_t<T>(C),
-                                         C.n_alloc);
-      else if (P.n_post >= 1)
-        dev::prolong_oct<T, true, kCG, true>(i, L.keys, L.blk, L.n, L.n_alloc, phi_t<T>(L), L.active, phi_t<T>(C),
-                                              C.n_alloc);
-      else
-        dev::prolong_oct<T, true, kCG>(i, L.keys, L.blk, L.n, L.n_alloc, phi_t<T>(L), L.active, phi_t<T>(C),
-                                        C.n_alloc);
-    }
-    if (!grid_sync(P)) return false;
-    if (!sweeps<T>(P, L, P.n_post, false, tid, nthr, phi_t<T>(L), g_t<T>(L))) return false;
-  }
-  return true;
+  return ascend<T>(all, mid - 1, 0);
 }
 
 // Top-level FP64 residual, per-patch norms into P.norm; MIXED also writes the
@@ -205,22 +406,34 @@ __device__ bool vcycle(const BatchPlan &P, bool zero_top, int64_t tid, int64_t n
 // V-cycle whose last operation on the top level is a colour-1 pass (the
 // colour-1 residuals are exactly zero and are not evaluated).
 template <bool MIXED, bool ZPHI, bool C1Z = false>
-__device__ void top_residual(const BatchPlan &P, double *acc_out, int64_t tid, int64_t nthr) {
-  const BLevel &L = P.lv[0];
-  const int64_t wbase = tid & ~(int64_t)31;
-  for (int64_t base = wbase; base < L.n; base += nthr) {
-    const int64_t i = base + (threadIdx.x & 31);
-    double acc = 0.0;
-    int p = -1;
-    if (i < L.n) {
-      p = __ldg(P.pid + i);
-      const double inv_s = MIXED ? 1.0 / __ldcg(P.s_emit + p) : 0.0;
-      acc = dev::resid_oct<double, true, false, MIXED, false, ZPHI, kCG, C1Z>(
-          i, L.nbr, L.phi, L.g, nullptr, L.n, L.n_alloc, nullptr, nullptr, nullptr, 0, 0, 0, L.g32, inv_s, nullptr,
-          0.0);
-    }
-    patch_add(acc_out, p, acc);
-  }
+__device__ __noinline__ void top_residual(const BatchPlan &P, double *acc_out) {
+  const BLevel L = P.lv[0];
+  const int32_t *pid = P.pid;
+  const double *s_emit = P.s_emit;
+  const Octs o = All{P}.units(0, 1);
+  PatchSum sum{acc_out};
+  const int lane = threadIdx.x & 31;
+  struct Idx {
+    dev::ResidIdx r;
+    int p;
+  };
+  // every lane of a warp takes part in each step (past the end: no patch)
+  for_octs<1>(Octs{o.a - lane, o.e, o.s},
+           [&](int64_t base) {
+             const int64_t i = base + lane;
+             if (i >= o.e) return Idx{{}, -1};
+             return Idx{dev::resid_idx<false>(i, L.nbr, nullptr, L.n, nullptr), __ldg(pid + i)};
+           },
+           [&](int64_t base, const Idx &x) {
+             double acc = 0.0;
+             if (x.p >= 0) {
+               const double inv_s = MIXED ? dev::inv_scale(__ldcg(s_emit + x.p)) : 0.0;
+               acc = dev::resid_oct_idx<double, true, false, MIXED, false, ZPHI, kCG, C1Z, true>(
+                   base + lane, x.r, L.phi, L.g, L.n, L.n_alloc, nullptr, nullptr, 0, 0, 0, L.g32, inv_s, nullptr, 0.0);
+             }
+             sum.add(x.p, acc);
+           });
+  sum.flush();
 }
 
 // Dirichlet ghosts of the top level from the parent's phi.
@@ -310,13 +523,13 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
   }
   for (int64_t p = tid; p < P.n_patches; p += nthr) {
     const double nr = __ldcg(P.norm + p);
-    P.s_emit[p] = nr > 0.0 ? sqrt(nr) : 1.0;
+    P.s_emit[p] = pow2_scale(sqrt(nr));
   }
   if (!grid_sync(P)) return false;
   if (MIXED) {  // the first FP32 right-hand side r0 / s
     for (int64_t t = tid; t < 8 * n; t += nthr) {
       const int64_t i = (t >> 2) % n;
-      T.g32[t] = (float)(T.g[t] / __ldcg(P.s_emit + __ldg(P.pid + i)));
+      T.g32[t] = dev::f32_scaled(T.g[t], dev::inv_scale(__ldcg(P.s_emit + __ldg(P.pid + i))));
     }
     if (!grid_sync(P)) return false;
   }
@@ -341,7 +554,7 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
       }
       if (MIXED) {
         P.s_acc[p] = __ldcg(P.s_emit + p);
-        P.s_emit[p] = nr > 0.0 ? sqrt(nr) : 1.0;
+        P.s_emit[p] = pow2_scale(sqrt(nr));
       }
       P.norm[p] = 0.0;
     }
@@ -363,9 +576,9 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
     // z = M r: one V-cycle from zero (FP64 on g = r, or FP32 on g32 = r / s)
     if (MIXED) {
       for (int k = 0; k < P.inner; ++k)
-        if (!vcycle<float>(P, k == 0, tid, nthr)) return false;
+        if (!vcycle<float>(P, k == 0)) return false;
     } else {
-      if (!vcycle<double>(P, true, tid, nthr)) return false;
+      if (!vcycle<double>(P, true)) return false;
     }
     // (z, r) and (z, q) per patch; q is the last iteration's L0 p
     for (int64_t base = wbase; base < n; base += nthr) {
@@ -449,14 +662,14 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
         pp = __ldg(P.pid + i);
         const double pq = __ldcg(P.pq + pp);
         const double al = (__ldcg(P.done + pp) || pq == 0.0) ? 0.0 : __ldcg(P.zr_old + pp) / pq;
-        const double inv_s = MIXED ? 1.0 / __ldcg(P.s_emit + pp) : 0.0;
+        const double inv_s = MIXED ? dev::inv_scale(__ldcg(P.s_emit + pp)) : 0.0;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           const int64_t k = at_phi(i, c, ps), gi = at_phi(i, c, gs);
           P.cx[k] += al * __ldcg(pn + k);
           const double rv = __ldcg(T.g + gi) - al * __ldcg(P.cq + k);
           T.g[gi] = rv;
-          if (MIXED) T.g32[gi] = (float)(rv * inv_s);
+          if (MIXED) T.g32[gi] = dev::f32_scaled(rv, inv_s);
           acc += rv * rv;
         }
       }
@@ -480,13 +693,13 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
 // until every patch reaches tol.
 template <bool MIXED>
 __device__ void stationary_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
-  const BLevel &T0 = P.lv[0];
+  const BLevel T0 = P.lv[0];
   for (int64_t p = tid; p < P.n_patches; p += nthr) {
     const double n0 = __ldcg(P.n0 + p);
-    P.s_emit[p] = n0 > 0.0 ? sqrt(n0) : 1.0;
+    P.s_emit[p] = pow2_scale(sqrt(n0));
   }
   if (!grid_sync(P)) return;
-  top_residual<MIXED, false>(P, P.norm, tid, nthr);
+  top_residual<MIXED, false>(P, P.norm);
   if (!grid_sync(P)) return;
   for (int cycle = 0;; ++cycle) {
     // per-patch test; unconverged patches counted in ctrl[2 + parity]
@@ -502,7 +715,7 @@ __device__ void stationary_solve(const BatchPlan &P, int64_t tid, int64_t nthr) 
       }
       if (MIXED) {
         P.s_acc[p] = __ldcg(P.s_emit + p);
-        P.s_emit[p] = nr > 0.0 ? sqrt(nr) : 1.0;
+        P.s_emit[p] = pow2_scale(sqrt(nr));
       }
       P.norm[p] = 0.0;
     }
@@ -523,28 +736,34 @@ __device__ void stationary_solve(const BatchPlan &P, int64_t tid, int64_t nthr) 
     if (tid == 0) P.ctrl[2 + ((cycle + 1) & 1)] = 0;
     if (MIXED) {
       for (int k = 0; k < P.inner; ++k)
-        if (!vcycle<float>(P, k == 0, tid, nthr)) return;
-      for (int64_t t = tid; t < 2 * T0.n; t += nthr) {  // phi64 += s_acc * e
-        const int pl = (int)(t / T0.n);
-        const int64_t i = t - pl * T0.n;
-        const double S = __ldcg(P.s_acc + __ldg(P.pid + i));
-        double v[4];
-        float w[4];
-        dev::load4<true>(T0.phi + (pl * T0.n_alloc + i) * 4, v);
-        dev::load4<true>(T0.phi32 + (pl * T0.n_alloc + i) * 4, w);
+        if (!vcycle<float>(P, k == 0)) return;
+      // phi64 += s_acc * e
+      for_octs<1>(All{P}.units(0, 1), [&](int64_t i) { return __ldg(P.pid + i); },
+                  [&](int64_t i, int p) {
+                    const double S = __ldcg(P.s_acc + p);
+                    double v[2][4];
+                    float w[2][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = fma(S, (double)w[q], v[q]);
-        dev::store4(T0.phi + (pl * T0.n_alloc + i) * 4, v);
-      }
+                    for (int pl = 0; pl < 2; ++pl) {
+                      dev::load4<kCG>(T0.phi + (pl * T0.n_alloc + i) * 4, v[pl]);
+                      dev::load4<kCG>(T0.phi32 + (pl * T0.n_alloc + i) * 4, w[pl]);
+                    }
+#pragma unroll
+                    for (int pl = 0; pl < 2; ++pl) {
+#pragma unroll
+                      for (int q = 0; q < 4; ++q) v[pl][q] = fma(S, dev::widen(w[pl][q]), v[pl][q]);
+                      dev::store4(T0.phi + (pl * T0.n_alloc + i) * 4, v[pl]);
+                    }
+                  });
       if (!grid_sync(P)) return;
-      top_residual<MIXED, false>(P, P.norm, tid, nthr);
+      top_residual<MIXED, false>(P, P.norm);
     } else {
-      if (!vcycle<double>(P, false, tid, nthr)) return;
+      if (!vcycle<double>(P, false)) return;
       const bool c1 = P.depth > 1 ? P.n_post >= 1 : P.n_pre + P.n_post >= 1;
       if (c1)
-        top_residual<false, false, true>(P, P.norm, tid, nthr);
+        top_residual<false, false, true>(P, P.norm);
       else
-        top_residual<false, false>(P, P.norm, tid, nthr);
+        top_residual<false, false>(P, P.norm);
     }
     if (!grid_sync(P)) return;
   }
@@ -562,7 +781,7 @@ __global__ void __launch_bounds__(512, 1) k_batch(const __grid_constant__ BatchP
     P.conv_at[p] = -1;
   }
   if (!grid_sync(P)) return;
-  top_residual<false, true>(P, P.n0, tid, nthr);  // ||f - L 0||^2 per patch
+  top_residual<false, true>(P, P.n0);  // ||f - L 0||^2 per patch
   if (!grid_sync(P)) return;
   if constexpr (KRYLOV)
     krylov_solve<MIXED>(P, tid, nthr);
@@ -606,6 +825,36 @@ __global__ void k_patch_check(const int32_t *__restrict__ pid, const int32_t *__
     const int32_t f = father[i];
     if (f >= 0 && cpid[f >> 3] != p) set_error(err, CMG_ERR_INVALID_ARG);
   }
+}
+
+// Whether blocks can work on their own patches on a coarse level: its octs
+// are in the patches' order, and its prolongation stays within the patch (the
+// check above sees face neighbours only).
+__global__ void k_patch_own(const int32_t *__restrict__ pid, const int32_t *__restrict__ father,
+                            const int32_t *__restrict__ blk, const int32_t *__restrict__ cpid, int64_t n, int64_t cn,
+                            int *mixed) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int32_t p = pid[i];
+  bool bad = i > 0 && pid[i - 1] > p;
+  if (cpid)
+    for (int t = 0; t < 8; ++t) {
+      const int32_t o = blk[t * n + i];
+      bad = bad || (o < cn && cpid[o] != p);
+    }
+  if (bad) *mixed = 1;
+}
+
+// starts[k]: the first oct of patch k (or of a later one), k = 0 .. n_patches
+__global__ void k_patch_starts(const int32_t *__restrict__ pid, int64_t n, int n_patches, int32_t *__restrict__ starts) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k > n_patches) return;
+  int64_t lo = 0, hi = n;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (pid[mid] < k) lo = mid + 1; else hi = mid;
+  }
+  starts[k] = (int32_t)lo;
 }
 
 }  // namespace
@@ -719,6 +968,43 @@ BatchPlan make_plan(cmg_batch *b, const cmg_solve_params *p) {
   return P;
 }
 
+// Deals the patches out to the blocks (contiguous ranges, about the same
+// number of octs) and finds the first level from which every block's octs
+// take at most two rounds of its threads in FP32, one in FP64: from there on
+// the blocks work on their own.
+void plan_own(cmg_batch *b, int grid, bool mixed, BatchPlan &P) {
+  P.split = P.depth;
+  const int n = b->n_patches;
+  std::vector<int> patch(grid + 1);  // the first patch of each block
+  for (int m = 1; m < P.depth && !b->starts.empty() && P.split == P.depth; ++m) {
+    const int32_t *st = b->starts.data() + (size_t)m * (n + 1);
+    const int64_t total = st[n];
+    int next = 0;
+    for (int k = 0; k < n; ++k) {
+      const int64_t mid = ((int64_t)st[k] + st[k + 1]) / 2;
+      const int to = (int)std::min<int64_t>(grid - 1, total > 0 ? mid * grid / total : 0);
+      for (; next <= to; ++next) patch[next] = k;
+    }
+    for (; next <= grid; ++next) patch[next] = n;
+    int64_t most = 0;
+    for (int q = 0; q < grid; ++q) most = std::max<int64_t>(most, st[patch[q + 1]] - st[patch[q]]);
+    if (most <= (mixed ? 2 : 1) * (int64_t)b->sched.threads) P.split = m;
+  }
+  if (P.split == P.depth) return;
+  const size_t count = (size_t)P.depth * (grid + 1);
+  std::vector<int32_t> first(count, 0);
+  for (int m = P.split; m < P.depth; ++m)
+    for (int q = 0; q <= grid; ++q) first[(size_t)m * (grid + 1) + q] = b->starts[(size_t)m * (n + 1) + patch[q]];
+  cudaStream_t s = b->lvl->ctx->stream;
+  if (b->first_cap < count) {
+    b->first = b->mem.alloc<int32_t>((int64_t)count);
+    b->first_cap = count;
+  }
+  CMG_CUDA(cudaMemcpyAsync(b->first, first.data(), count * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  CMG_CUDA(cudaStreamSynchronize(s));
+  P.first = b->first;
+}
+
 // CG vectors and per-patch scalars (krylov = 1), allocated on first use
 void ensure_cg(cmg_batch *b) {
   if (b->cg) return;
@@ -740,6 +1026,7 @@ void record(cmg_batch *b, const cmg_solve_params *p) {
   const bool mixed = p->precision == CMG_PREC_MIXED, krylov = p->krylov == 1;
   BatchPlan P = make_plan(b, p);
   const int grid = grid_size(b, mixed, krylov);
+  plan_own(b, grid, mixed, P);
   if (!ctx->cap_stream) {
     CMG_CUDA(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
     CMG_CUDA(cudaStreamCreateWithFlags(&ctx->cap_stream2, cudaStreamNonBlocking));
@@ -862,6 +1149,22 @@ void batch_create(cmg_level *L, const int64_t *offsets, int n_patches, cmg_batch
                                                                   ctx->d_err);
     }
     CMG_CUDA(cudaGetLastError());
+    const size_t depth = L->mg.size();
+    int32_t *d_starts = b->mem.alloc<int32_t>((int64_t)depth * (n_patches + 1), true, s);
+    int32_t *d_mixed = b->mem.alloc<int32_t>(1, true, s);
+    for (size_t m = 1; m < depth; ++m) {
+      const MgLev &g = L->mg[m];
+      const bool has_c = m + 1 < depth;
+      k_patch_own<<<blocks_for(g.n), kThreads, 0, s>>>(b->pid[m], g.father, g.blk, has_c ? b->pid[m + 1] : nullptr, g.n,
+                                                       has_c ? L->mg[m + 1].n : 0, d_mixed);
+      k_patch_starts<<<blocks_for(n_patches + 1), kThreads, 0, s>>>(b->pid[m], g.n, n_patches,
+                                                                    d_starts + m * (n_patches + 1));
+    }
+    CMG_CUDA(cudaGetLastError());
+    int mixed = 0;
+    b->starts.resize(depth * (n_patches + 1));
+    CMG_CUDA(cudaMemcpyAsync(b->starts.data(), d_starts, b->starts.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    CMG_CUDA(cudaMemcpyAsync(&mixed, d_mixed, sizeof(int), cudaMemcpyDeviceToHost, s));
     int err = 0;
     CMG_CUDA(cudaMemcpyAsync(&err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
     CMG_CUDA(cudaStreamSynchronize(s));
@@ -869,6 +1172,7 @@ void batch_create(cmg_level *L, const int64_t *offsets, int n_patches, cmg_batch
       CMG_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), s));
       throw Error(CMG_ERR_INVALID_ARG, "patches are not independent: a neighbour link joins two patches");
     }
+    if (mixed) b->starts.clear();
     b->pstate = b->mem.alloc<double>(5 * (int64_t)n_patches, true, s);
     b->conv_at = b->mem.alloc<int32_t>(n_patches, true, s);
     b->ctrl = b->mem.alloc<int>(8, true, s);

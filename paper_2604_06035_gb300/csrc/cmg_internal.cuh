@@ -354,6 +354,11 @@ struct cmg_batch {
   cmg_batch_schedule sched = {256, 2, 2, 2, 1};
   long long spin_budget = 2000000000ll;
   std::vector<int32_t *> pid;  // patch of each oct, per MG level
+  // [depth][n_patches + 1] first oct of each patch on the coarse levels; empty
+  // where blocks cannot work on their own patches there (batch.cu)
+  std::vector<int32_t> starts;
+  int32_t *first = nullptr;    // first oct of each block of the recorded grid, per MG level
+  size_t first_cap = 0;
   double *pstate = nullptr;    // n0, norm, s_emit, s_acc, rel: 5 x n_patches
   int32_t *conv_at = nullptr;
   int *ctrl = nullptr;         // 8 ints
