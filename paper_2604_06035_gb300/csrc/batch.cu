@@ -62,7 +62,7 @@ struct BatchPlan {
   unsigned *bar;  // grid barrier word
   // conjugate gradients (krylov = 1): top-level vectors in the phi layout
   // ([2][n_alloc][4]; gsave in the g layout) and per-patch scalars
-  double *cx, *cp0, *cp1, *cq, *gsave;
+  double *cx, *cp, *cq, *gsave;
   double *zr, *zq, *zr_old, *beta, *pq, *alpha;
   int32_t *done;
 };
@@ -179,16 +179,6 @@ struct PatchSum {
     acc = 0.0;
   }
 };
-
-// The FP32 right-hand sides' scale for a norm: the power of two of its binade
-// (products with it are exact), itself if infinite, else 1.
-__device__ __forceinline__ double pow2_scale(double v) {
-  if (!(v > 0.0)) return 1.0;
-  if (v == INFINITY) return v;
-  int e;
-  (void)frexp(v, &e);
-  return ldexp(1.0, e - 1);
-}
 
 template <typename T>
 __device__ __forceinline__ T *phi_t(const BLevel &L) {
@@ -466,50 +456,61 @@ __device__ void fill_top_ghosts(const BatchPlan &P, int64_t tid, int64_t nthr) {
 // (pcg.cu) with a separate alpha and beta for every patch.  A patch that has
 // reached tol keeps alpha = beta = 0 (frozen) while the others iterate.
 
-__device__ __forceinline__ int64_t at_phi(int64_t o, int c, int64_t ps) {
-  return (int64_t)cell_parity(c) * ps + o * 4 + (c >> 1);
+// z on plane pl of oct i of a patch: the FP64 V-cycle leaves z in phi; the
+// FP32 one leaves e = z / s in phi32
+template <bool MIXED>
+__device__ __forceinline__ void load_z(const BLevel &T, int64_t i, int pl, double s, double z[4]) {
+  const int64_t k = (pl * T.n_alloc + i) * 4;
+  if constexpr (MIXED) {
+    float e[4];
+    dev::load4<kCG>(T.phi32 + k, e);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) z[q] = s * dev::widen(e[q]);
+  } else {
+    dev::load4<kCG>(T.phi + k, z);
+  }
 }
 
-// z at phi-layout index k of a cell of patch p: the FP64 V-cycle leaves z in
-// phi; the FP32 one leaves e = z / s_acc in phi32
-template <bool MIXED>
-__device__ __forceinline__ double zval(const BatchPlan &P, int64_t k, double s) {
-  if constexpr (MIXED) return s * (double)__ldcg(P.lv[0].phi32 + k);
-  else return __ldcg(P.lv[0].phi + k);
+// The level-wide passes of the iteration: body(i, patch) for every oct of the
+// thread; per-patch sums of what it returns.
+template <class Body>
+__device__ __forceinline__ void patch_pass(const BatchPlan &P, double *sum0, double *sum1, Body body) {
+  const Octs o = All{P}.units(0, 1);
+  const int lane = threadIdx.x & 31;
+  const int32_t *pid = P.pid;
+  PatchSum s0{sum0}, s1{sum1};
+  for_octs<1>(Octs{o.a - lane, o.e, o.s}, [&](int64_t base) { return base + lane < o.e ? __ldg(pid + base + lane) : -1; },
+              [&](int64_t base, int p) {
+                double v[2] = {0.0, 0.0};
+                if (p >= 0) body(base + lane, p, v);
+                if (sum0) s0.add(p, v[0]);
+                if (sum1) s1.add(p, v[1]);
+              });
+  if (sum0) s0.flush();
+  if (sum1) s1.flush();
 }
 
 template <bool MIXED>
 __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
-  const BLevel &T = P.lv[0];
-  const int64_t n = T.n, ps = T.n_alloc * 4, gs = n * 4;
-  const int64_t wbase = tid & ~(int64_t)31;
+  const BLevel T = P.lv[0];
+  const int64_t n = T.n, na = T.n_alloc, ps = na * 4;
   // r0 = f - L phi0 (Dirichlet ghosts) in place of g (saved), x = phi0, ||r0||^2
-  for (int64_t base = wbase; base < n; base += nthr) {
-    const int64_t i = base + (threadIdx.x & 31);
-    double acc = 0.0;
-    int pp = -1;
-    if (i < n) {
-      pp = __ldg(P.pid + i);
+  patch_pass(P, P.norm, nullptr, [&](int64_t i, int, double *sum) {
+    double ph[2][4], lp[2][4], gv[4], rv[4];
+    dev::apply_oct<kCG>(i, T.nbr, T.phi, n, na, ph, lp);
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        double sum = 0.0;
+    for (int pl = 0; pl < 2; ++pl) {
+      dev::load4<kCG>(T.g + (pl * n + i) * 4, gv);
 #pragma unroll
-        for (int d = 0; d < 6; ++d) {
-          const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
-          const int64_t o = (((c >> a) & 1) != side) ? i : (int64_t)__ldg(T.nbr + d * n + i);
-          sum += __ldcg(T.phi + at_phi(o, c2, ps));
-        }
-        const int64_t gi = at_phi(i, c, gs), k = at_phi(i, c, ps);
-        const double gv = __ldcg(T.g + gi), ph = __ldcg(T.phi + k);
-        const double v = fma(sum, 1.0 / 6.0, gv) - ph;
-        P.gsave[gi] = gv;
-        T.g[gi] = v;
-        P.cx[k] = ph;
-        acc += v * v;
+      for (int q = 0; q < 4; ++q) {
+        rv[q] = gv[q] - lp[pl][q];
+        sum[0] = fma(rv[q], rv[q], sum[0]);
       }
+      dev::store4(P.gsave + (pl * n + i) * 4, gv);
+      dev::store4(T.g + (pl * n + i) * 4, rv);
+      dev::store4(P.cx + (pl * na + i) * 4, ph[pl]);
     }
-    patch_add(P.norm, pp, acc);
-  }
+  });
   for (int64_t p = tid; p < P.n_patches; p += nthr) {
     P.zr[p] = P.zq[p] = P.zr_old[p] = P.beta[p] = P.pq[p] = P.alpha[p] = 0.0;
     P.done[p] = 0;
@@ -523,7 +524,7 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
   }
   for (int64_t p = tid; p < P.n_patches; p += nthr) {
     const double nr = __ldcg(P.norm + p);
-    P.s_emit[p] = pow2_scale(sqrt(nr));
+    P.s_emit[p] = dev::pow2_scale(sqrt(nr));
   }
   if (!grid_sync(P)) return false;
   if (MIXED) {  // the first FP32 right-hand side r0 / s
@@ -533,19 +534,13 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
     }
     if (!grid_sync(P)) return false;
   }
-  int cur = 0;  // direction buffer written this iteration
   for (int cycle = 0;; ++cycle) {
-    // stop test on ||r||; alpha of the last step kept for the next beta
+    // stop test on ||r||
     for (int64_t p = tid; p < P.n_patches; p += nthr) {
       const double n0 = __ldcg(P.n0 + p), nr = __ldcg(P.norm + p);
       const double rel = n0 > 0.0 ? sqrt(nr / n0) : 0.0;
       P.rel[p] = rel;
       if (!(rel == rel) || isinf(rel)) atomicCAS(P.ctrl, 0, CMG_ERR_DIVERGED);
-      const int was_done = __ldcg(P.done + p);
-      if (cycle > 0) {
-        const double pq = __ldcg(P.pq + p), zo = __ldcg(P.zr_old + p);
-        P.alpha[p] = (was_done || pq == 0.0) ? 0.0 : zo / pq;
-      }
       if (rel <= P.tol) {
         if (__ldcg(P.conv_at + p) < 0) P.conv_at[p] = cycle;
         P.done[p] = 1;
@@ -554,7 +549,7 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
       }
       if (MIXED) {
         P.s_acc[p] = __ldcg(P.s_emit + p);
-        P.s_emit[p] = pow2_scale(sqrt(nr));
+        P.s_emit[p] = dev::pow2_scale(sqrt(nr));
       }
       P.norm[p] = 0.0;
     }
@@ -581,24 +576,21 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
       if (!vcycle<double>(P, true)) return false;
     }
     // (z, r) and (z, q) per patch; q is the last iteration's L0 p
-    for (int64_t base = wbase; base < n; base += nthr) {
-      const int64_t i = base + (threadIdx.x & 31);
-      double a = 0.0, b = 0.0;
-      int pp = -1;
-      if (i < n) {
-        pp = __ldg(P.pid + i);
-        const double sz = MIXED ? __ldcg(P.s_acc + pp) : 1.0;
+    patch_pass(P, P.zr, P.zq, [&](int64_t i, int pp, double *sum) {
+      const double sz = MIXED ? __ldcg(P.s_acc + pp) : 1.0;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int64_t k = at_phi(i, c, ps);
-          const double z = zval<MIXED>(P, k, sz);
-          a += z * __ldcg(T.g + at_phi(i, c, gs));
-          b += z * __ldcg(P.cq + k);
+      for (int pl = 0; pl < 2; ++pl) {
+        double z[4], r[4], qv[4];
+        load_z<MIXED>(T, i, pl, sz, z);
+        dev::load4<kCG>(T.g + (pl * n + i) * 4, r);
+        dev::load4<kCG>(P.cq + (pl * na + i) * 4, qv);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          sum[0] = fma(z[q], r[q], sum[0]);
+          sum[1] = fma(z[q], qv[q], sum[1]);
         }
       }
-      patch_add(P.zr, pp, a);
-      patch_add(P.zq, pp, b);
-    }
+    });
     if (!grid_sync(P)) return false;
     // beta = -alpha (z', q) / (z, r)_old (0 on the first iteration and once frozen)
     for (int64_t p = tid; p < P.n_patches; p += nthr) {
@@ -611,72 +603,70 @@ __device__ bool krylov_solve(const BatchPlan &P, int64_t tid, int64_t nthr) {
       P.pq[p] = 0.0;
     }
     if (!grid_sync(P)) return false;
-    // p = z + beta p_old into the other direction buffer (ghost and zero octs
-    // stay zero), then q = L0 p and (p, q) per patch (neighbours share the
-    // patch).  Two passes: forming the neighbours' p on the fly would cost six
-    // more FP64 FMAs per cell than the extra pass costs bandwidth.
-    double *pn = cur ? P.cp1 : P.cp0;
-    const double *po = cur ? P.cp0 : P.cp1;
-    for (int64_t i = tid; i < n; i += nthr) {
-      const int pp = __ldg(P.pid + i);
+    // p = z + beta p (its ghost and zero octs stay zero), then q = L0 p and
+    // (p, q) per patch (neighbours share the patch).  Two passes: forming the
+    // neighbours' p on the fly would cost six more FP64 FMAs per cell than the
+    // extra pass costs bandwidth.
+    patch_pass(P, nullptr, nullptr, [&](int64_t i, int pp, double *) {
       const double bt = __ldcg(P.beta + pp), sz = MIXED ? __ldcg(P.s_acc + pp) : 1.0;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int64_t k = at_phi(i, c, ps);
-        pn[k] = fma(bt, __ldcg(po + k), zval<MIXED>(P, k, sz));
+      for (int pl = 0; pl < 2; ++pl) {
+        double z[4], pv[4];
+        double *at = P.cp + (pl * na + i) * 4;
+        load_z<MIXED>(T, i, pl, sz, z);
+        dev::load4<kCG>(at, pv);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) pv[q] = fma(bt, pv[q], z[q]);
+        dev::store4(at, pv);
       }
-    }
+    });
     if (!grid_sync(P)) return false;
-    for (int64_t base = wbase; base < n; base += nthr) {
-      const int64_t i = base + (threadIdx.x & 31);
-      double acc = 0.0;
-      int pp = -1;
-      if (i < n) {
-        pp = __ldg(P.pid + i);
+    patch_pass(P, P.pq, nullptr, [&](int64_t i, int, double *sum) {
+      double pv[2][4], qv[2][4];
+      dev::apply_oct<kCG>(i, T.nbr, P.cp, n, na, pv, qv);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int64_t k = at_phi(i, c, ps);
-          const double pv = __ldcg(pn + k);
-          double sum = 0.0;
+      for (int pl = 0; pl < 2; ++pl) {
 #pragma unroll
-          for (int d = 0; d < 6; ++d) {
-            const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
-            const int64_t o = (((c >> a) & 1) != side) ? i : (int64_t)__ldg(T.nbr + d * n + i);
-            sum += __ldcg(pn + at_phi(o, c2, ps));
-          }
-          const double qv = pv - sum * (1.0 / 6.0);
-          P.cq[k] = qv;
-          acc += pv * qv;
-        }
+        for (int q = 0; q < 4; ++q) sum[0] = fma(pv[pl][q], qv[pl][q], sum[0]);
+        dev::store4(P.cq + (pl * na + i) * 4, qv[pl]);
       }
-      patch_add(P.pq, pp, acc);
-    }
+    });
     if (!grid_sync(P)) return false;
     // alpha = (z, r) / (p, q); x += alpha p; r -= alpha q; ||r||^2 per patch;
-    // MIXED: the next FP32 right-hand side r / s
-    for (int64_t base = wbase; base < n; base += nthr) {
-      const int64_t i = base + (threadIdx.x & 31);
-      double acc = 0.0;
-      int pp = -1;
-      if (i < n) {
-        pp = __ldg(P.pid + i);
-        const double pq = __ldcg(P.pq + pp);
-        const double al = (__ldcg(P.done + pp) || pq == 0.0) ? 0.0 : __ldcg(P.zr_old + pp) / pq;
-        const double inv_s = MIXED ? dev::inv_scale(__ldcg(P.s_emit + pp)) : 0.0;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int64_t k = at_phi(i, c, ps), gi = at_phi(i, c, gs);
-          P.cx[k] += al * __ldcg(pn + k);
-          const double rv = __ldcg(T.g + gi) - al * __ldcg(P.cq + k);
-          T.g[gi] = rv;
-          if (MIXED) T.g32[gi] = dev::f32_scaled(rv, inv_s);
-          acc += rv * rv;
-        }
-      }
-      patch_add(P.norm, pp, acc);
+    // MIXED: the next FP32 right-hand side r / s.  alpha is formed once per
+    // patch: an FP64 division costs as much as ten FMAs.
+    for (int64_t p = tid; p < P.n_patches; p += nthr) {
+      const double pq = __ldcg(P.pq + p);
+      P.alpha[p] = (__ldcg(P.done + p) || pq == 0.0) ? 0.0 : __ldcg(P.zr_old + p) / pq;
     }
     if (!grid_sync(P)) return false;
-    cur ^= 1;
+    patch_pass(P, P.norm, nullptr, [&](int64_t i, int pp, double *sum) {
+      const double al = __ldcg(P.alpha + pp), inv_s = MIXED ? dev::inv_scale(__ldcg(P.s_emit + pp)) : 0.0;
+#pragma unroll
+      for (int pl = 0; pl < 2; ++pl) {
+        const int64_t k = (pl * na + i) * 4, gk = (pl * n + i) * 4;
+        double xv[4], pv[4], rv[4], qv[4];
+        dev::load4<kCG>(P.cx + k, xv);
+        dev::load4<kCG>(P.cp + k, pv);
+        dev::load4<kCG>(T.g + gk, rv);
+        dev::load4<kCG>(P.cq + k, qv);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          xv[q] = fma(al, pv[q], xv[q]);
+          rv[q] = fma(-al, qv[q], rv[q]);
+          sum[0] = fma(rv[q], rv[q], sum[0]);
+        }
+        dev::store4(P.cx + k, xv);
+        dev::store4(T.g + gk, rv);
+        if (MIXED) {
+          float w[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) w[q] = dev::f32_scaled(rv[q], inv_s);
+          dev::store4(T.g32 + gk, w);
+        }
+      }
+    });
+    if (!grid_sync(P)) return false;
   }
   // wrap-up: phi = x, the source restored, the coarse-fine ghosts refilled
   for (int64_t t = tid; t < 8 * n; t += nthr) {
@@ -696,7 +686,7 @@ __device__ void stationary_solve(const BatchPlan &P, int64_t tid, int64_t nthr) 
   const BLevel T0 = P.lv[0];
   for (int64_t p = tid; p < P.n_patches; p += nthr) {
     const double n0 = __ldcg(P.n0 + p);
-    P.s_emit[p] = pow2_scale(sqrt(n0));
+    P.s_emit[p] = dev::pow2_scale(sqrt(n0));
   }
   if (!grid_sync(P)) return;
   top_residual<MIXED, false>(P, P.norm);
@@ -715,7 +705,7 @@ __device__ void stationary_solve(const BatchPlan &P, int64_t tid, int64_t nthr) 
       }
       if (MIXED) {
         P.s_acc[p] = __ldcg(P.s_emit + p);
-        P.s_emit[p] = pow2_scale(sqrt(nr));
+        P.s_emit[p] = dev::pow2_scale(sqrt(nr));
       }
       P.norm[p] = 0.0;
     }
@@ -953,9 +943,8 @@ BatchPlan make_plan(cmg_batch *b, const cmg_solve_params *p) {
   if (b->cg) {
     const int64_t nv = 8 * L->mg[0].n_alloc;
     P.cx = b->cg;
-    P.cp0 = P.cx + nv;
-    P.cp1 = P.cp0 + nv;
-    P.cq = P.cp1 + nv;
+    P.cp = P.cx + nv;
+    P.cq = P.cp + nv;
     P.gsave = P.cq + nv;
     P.zr = P.gsave + 8 * L->mg[0].n;
     P.zq = P.zr + n;
@@ -1011,13 +1000,13 @@ void ensure_cg(cmg_batch *b) {
   cmg_level *L = b->lvl;
   const int64_t nv = 8 * L->mg[0].n_alloc;
   // b->cg (the "allocated" mark) is set last
-  double *cg = b->mem.alloc<double>(4 * nv + 8 * L->mg[0].n + 6 * (int64_t)b->n_patches, true, L->ctx->stream);
+  double *cg = b->mem.alloc<double>(3 * nv + 8 * L->mg[0].n + 6 * (int64_t)b->n_patches, true, L->ctx->stream);
   b->cg_done = b->mem.alloc<int32_t>(b->n_patches, true, L->ctx->stream);
   CMG_CUDA(cudaStreamSynchronize(L->ctx->stream));
   b->cg = cg;
 }
 
-// Records: clear control words (and the CG direction buffers), the
+// Records: clear control words (and the CG direction and q), the
 // cooperative persistent kernel, copy of the control words to pinned host
 // memory.
 void record(cmg_batch *b, const cmg_solve_params *p) {
@@ -1037,8 +1026,8 @@ void record(cmg_batch *b, const cmg_solve_params *p) {
   try {
     CMG_CUDA(cudaMemsetAsync(b->ctrl, 0, 8 * sizeof(int), s));
     CMG_CUDA(cudaMemsetAsync(b->bar, 0, 2 * sizeof(unsigned), s));
-    if (krylov)  // both direction buffers and q start at zero (finite) every solve
-      CMG_CUDA(cudaMemsetAsync(P.cp0, 0, sizeof(double) * 3 * 8 * L->mg[0].n_alloc, s));
+    if (krylov)  // the direction and q start at zero (finite) every solve
+      CMG_CUDA(cudaMemsetAsync(P.cp, 0, sizeof(double) * 2 * 8 * L->mg[0].n_alloc, s));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(b->sched.threads);

@@ -331,6 +331,15 @@ __device__ __forceinline__ double widen(float x) {
   if (m - 0x00800000u >= 0x7F000000u && m != 0) return (double)x;  // subnormal, infinite, NaN
   return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(b << 29));
 }
+// The FP32 right-hand sides' scale for a norm: the power of two of its binade
+// (products with it are exact), itself if infinite, else 1.
+__device__ __forceinline__ double pow2_scale(double v) {
+  if (!(v > 0.0)) return 1.0;
+  if (v == INFINITY) return v;
+  int e;
+  (void)frexp(v, &e);
+  return ldexp(1.0, e - 1);
+}
 // 1 / s: exact and without the FP64 pipe's ten-odd instructions for a normal
 // power of two.
 __device__ __forceinline__ double inv_scale(double s) {
@@ -479,6 +488,54 @@ __device__ __forceinline__ double resid_oct(int64_t i, const int32_t *__restrict
   return resid_oct_idx<T, NORM, RESTRICT, EMIT, ROUT, ZPHI, CG, C1Z, WIDE>(i, resid_idx<RESTRICT>(i, nbr, active, n, father),
                                                                 phi, g, n, n_alloc, cg, cphi, cn, cn_alloc,
                                                                 zero_cphi, g32, inv_s, rout, rscale);
+}
+
+// p - (sum of the six neighbours of p) / 6 on an oct: pv the oct's own values,
+// qv the result, by planes; missing neighbours are ghost octs or the zero oct
+// of p ([2][n_alloc][4]).  Whole planes and the integer sum, as above.
+template <bool CG>
+__device__ __forceinline__ void apply_oct(int64_t i, const int32_t *__restrict__ nbr, const double *p, int64_t n,
+                                          int64_t n_alloc, double pv[2][4], double qv[2][4]) {
+  int32_t nb[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) nb[d] = __ldg(nbr + d * n + i);
+  load4<CG>(p + i * 4, pv[0]);
+  load4<CG>(p + (n_alloc + i) * 4, pv[1]);
+#pragma unroll
+  for (int pl = 0; pl < 2; ++pl) {
+    double nv[6][4];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      const double *at = p + ((1 - pl) * n_alloc + (int64_t)nb[d]) * 4;
+      if (CG) load4<CG>(at, nv[d]);
+      else load_oct(at, nv[d]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = plane_cell(pl, q);
+      double v[6];
+#pragma unroll
+      for (int d = 0; d < 6; ++d) {
+        const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
+        v[d] = ((c >> a) & 1) != side ? pv[1 - pl][c2 >> 1] : nv[d][c2 >> 1];
+      }
+      qv[pl][q] = fma(fixed_sum<6>(v), -1.0 / 6.0, pv[pl][q]);
+    }
+  }
+}
+// The same for cell c of oct i.
+__device__ __forceinline__ void apply_cell(int64_t i, int c, const int32_t *__restrict__ nbr, const double *p, int64_t n,
+                                           int64_t n_alloc, double &pv, double &qv) {
+  const int pl = cell_parity(c);
+  double v[6];
+  pv = p[(pl * n_alloc + i) * 4 + (c >> 1)];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const int a = d >> 1, side = d & 1, c2 = c ^ (1 << a);
+    const int64_t o = (((c >> a) & 1) != side) ? i : (int64_t)__ldg(nbr + d * n + i);
+    v[d] = p[((1 - pl) * n_alloc + o) * 4 + (c2 >> 1)];
+  }
+  qv = fma(fixed_sum<6>(v), -1.0 / 6.0, pv);
 }
 
 // resid_oct<NORM = false, RESTRICT = true> with one thread per cell: lane k
