@@ -331,7 +331,11 @@ struct cmg_level {
   bool has32 = false;
   // schedule: MG levels with at most this many octs (and all coarser ones) run
   // in one "tail" launch (tail.cu); 0 = one launch per operation everywhere
-  int64_t tail_octs_fp64 = 32768;
+  // FP64: what one CTA takes (tail.cu); larger levels as launches with a thread
+  // per cell beat the grid tail (tail up to 64 / 1024 / 4096 / 32768 octs: 32^3
+  // solve 740 / 812 / 810 / 807 us, 128^3 two-level 3670 / 3750 / 3810 / 3900 us,
+  // 64^3 two-level CG 1980 / 2050 / 2064 / 2116 us)
+  int64_t tail_octs_fp64 = 64;
   int64_t tail_octs_fp32 = 2048;
   // colour passes of lexicographic full periodic levels in the shared-memory
   // brick kernel (brick.cu): 0 = never, 1 = FP32 passes (default; the FP64

@@ -298,6 +298,48 @@ __device__ __forceinline__ void sweep_cell(int64_t i, int q, const int32_t *__re
   dst[i * 4 + q] = out;
 }
 
+// sweep_cell with what a run of passes over a level reads again each time
+// (index data, right-hand sides) kept in registers: slot q of both planes of
+// oct i.  The two cells differ in their x bit alone, so they share their y and
+// z neighbours.
+struct CellRun {
+  int32_t xn[2], yn, zn;  // neighbour octs the two cells look out to
+  unsigned m;             // their activity, by plane
+  double g[2];
+};
+template <bool MASK>
+__device__ __forceinline__ CellRun cell_run(int64_t i, int q, const int32_t *__restrict__ nbr, const double *g,
+                                            const uint8_t *__restrict__ active, int64_t n) {
+  CellRun r;
+  r.yn = __ldg(nbr + (2 + (q & 1)) * n + i);
+  r.zn = __ldg(nbr + (4 + (q >> 1)) * n + i);
+  const unsigned m = MASK ? __ldg(active + i) : 0xFFu;
+  r.m = 0;
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const int c = plane_cell(p, q);
+    r.xn[p] = __ldg(nbr + (c & 1) * n + i);
+    r.m |= ((m >> c) & 1u) << p;
+    r.g[p] = g[(p * n + i) * 4 + q];
+  }
+  return r;
+}
+template <int P, bool ZERO, bool MASK>
+__device__ __forceinline__ void sweep_cell_run(int64_t i, int q, const CellRun &r, const double *src, double *dst) {
+  double out = r.g[P];
+  if (!ZERO) {
+    // the cell's slots one step along x, y, z are q, q ^ 1, q ^ 2
+    const double *own = src + i * 4;
+    const double ze = src[(int64_t)r.zn * 4 + (q ^ 2)], zi = own[q ^ 2];
+    const bool up = (q & 2) != 0;  // the outer z neighbour is the one above
+    const double v[6] = {own[q], src[(int64_t)r.xn[P] * 4 + q], own[q ^ 1], src[(int64_t)r.yn * 4 + (q ^ 1)],
+                         up ? zi : ze, up ? ze : zi};
+    out = fma(nbsum6(v), 1.0 / 6.0, out);
+  }
+  if (MASK && !((r.m >> P) & 1u)) out = 0.0;
+  dst[i * 4 + q] = out;
+}
+
 // Residual of oct i: d = fma(s, 1/6, g) - phi per cell, r = (-6 / h^2) d.
 // Returns the sum of d^2 over the oct (NORM; accumulated in FP64 for FP64
 // data, in FP32 within the oct for FP32 data, whose FP64 conversions would

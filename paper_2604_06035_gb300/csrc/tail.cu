@@ -139,8 +139,39 @@ __device__ void colour_pass(const TailLevel &L, int P, bool zero, const Map &map
     pass<T, true, CG>(L, P, zero, map);
 }
 
+// A run of sweeps over a level with at most one cell pair per thread: index
+// data and right-hand sides stay in registers.  Read in every pass, after a
+// barrier that empties L1, the indices put a second L2 round trip in front of
+// the neighbours' values.
+template <bool MASK, class Map, class Sync>
+__device__ void cell_sweeps(const TailLevel &L, int n_sweeps, bool zero_first, const Map &map, Sync &sync) {
+  const Span su = map.units(L.n, 4);
+  const bool on = su.a < su.e;
+  const int64_t i = su.a >> 2;
+  const int q = (int)(su.a & 3);
+  double *p0 = static_cast<double *>(L.phi), *p1 = p0 + L.n_alloc * 4;
+  dev::CellRun r = {};
+  if (on) r = dev::cell_run<MASK>(i, q, L.nbr, static_cast<const double *>(L.g), L.active, L.n);
+  for (int k = 0; k < n_sweeps; ++k) {
+    if (on) {
+      if (zero_first && k == 0) dev::sweep_cell_run<0, true, MASK>(i, q, r, p1, p0);
+      else dev::sweep_cell_run<0, false, MASK>(i, q, r, p1, p0);
+    }
+    sync();
+    if (on) dev::sweep_cell_run<1, false, MASK>(i, q, r, p0, p1);
+    sync();
+  }
+}
+
 template <typename T, bool CG, class Map, class Sync>
 __device__ void sweeps(const TailLevel &L, int n_sweeps, bool zero_first, const Map &map, Sync &sync) {
+  if constexpr (sizeof(T) == 8 && !CG) {
+    if (per_cell<T>(map, L.n)) {
+      if (L.all_active) cell_sweeps<false>(L, n_sweeps, zero_first, map, sync);
+      else cell_sweeps<true>(L, n_sweeps, zero_first, map, sync);
+      return;
+    }
+  }
   for (int k = 0; k < n_sweeps; ++k) {
     colour_pass<T, CG>(L, 0, zero_first && k == 0, map);
     sync();
