@@ -6,9 +6,11 @@
 // level's keys), so the level's hash table, neighbour cache, ghost octs and
 // multigrid hierarchy serve all of them; isolation between patches is
 // checked at build time on every MG level.  The persistent kernel walks the
-// whole V-cycle schedule with grid-stride loops over octs and a grid barrier
-// between dependent operations; per-patch residual norms are accumulated
-// with warp-aggregated atomics, and the stopping test runs on the device.
+// whole V-cycle schedule: the large levels with grid-stride loops over octs
+// and a grid barrier between dependent operations, the coarse ones block by
+// block, each on its own patches with block barriers.  Per-patch residual
+// norms are accumulated with warp-aggregated atomics, and the stopping test
+// runs on the device.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -820,9 +822,8 @@ __global__ void k_patch_check(const int32_t *__restrict__ pid, const int32_t *__
 // Whether blocks can work on their own patches on a coarse level: its octs
 // are in the patches' order, and its prolongation stays within the patch (the
 // check above sees face neighbours only).
-__global__ void k_patch_own(const int32_t *__restrict__ pid, const int32_t *__restrict__ father,
-                            const int32_t *__restrict__ blk, const int32_t *__restrict__ cpid, int64_t n, int64_t cn,
-                            int *mixed) {
+__global__ void k_patch_own(const int32_t *__restrict__ pid, const int32_t *__restrict__ blk,
+                            const int32_t *__restrict__ cpid, int64_t n, int64_t cn, int *mixed) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int32_t p = pid[i];
@@ -1144,7 +1145,7 @@ void batch_create(cmg_level *L, const int64_t *offsets, int n_patches, cmg_batch
     for (size_t m = 1; m < depth; ++m) {
       const MgLev &g = L->mg[m];
       const bool has_c = m + 1 < depth;
-      k_patch_own<<<blocks_for(g.n), kThreads, 0, s>>>(b->pid[m], g.father, g.blk, has_c ? b->pid[m + 1] : nullptr, g.n,
+      k_patch_own<<<blocks_for(g.n), kThreads, 0, s>>>(b->pid[m], g.blk, has_c ? b->pid[m + 1] : nullptr, g.n,
                                                        has_c ? L->mg[m + 1].n : 0, d_mixed);
       k_patch_starts<<<blocks_for(n_patches + 1), kThreads, 0, s>>>(b->pid[m], g.n, n_patches,
                                                                     d_starts + m * (n_patches + 1));

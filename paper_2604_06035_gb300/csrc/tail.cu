@@ -1,7 +1,7 @@
 // tail.cu -- the small multigrid levels of a V-cycle in one launch.
 //
-// Below a few ten thousand octs a level's work no longer fills the GPU and
-// each operation would cost a full kernel launch.  The tail kernel runs every
+// Small levels' work does not fill the GPU and each operation would cost a
+// full kernel launch.  The tail kernel runs every
 // operation of the V-cycle from MG level m0 down to the coarsest and back up:
 // pre-smoothing, residual + restriction, the coarsest solve (exact 2^3
 // transform or red-black sweeps), prolongation and post-smoothing.
