@@ -12,7 +12,7 @@
 //     (ld.global.cg), since another CTA may have written the data.  Levels
 //     small enough for one SM run inside the same launch on CTA 0 alone,
 //     with block barriers, while the others wait at the next grid barrier.
-//   * Single-CTA tail: when even the first tail level fits one SM, one CTA of
+//   * Single-CTA tail: when even the first tail level fits one SM, one CTA of 512 or
 //     1024 threads with block barriers and L1 loads.
 // The arithmetic is the same per-oct code as the one-launch-per-operation
 // path (oct_ops.cuh), so every schedule gives the same results.
@@ -309,7 +309,11 @@ struct GridSync {
   __device__ void operator()() { dev::grid_barrier(bar, err, budget); }
 };
 
-constexpr int kTailThreads1 = 1024;
+// One CTA: in FP64 a thread for each of the 8 cells of 64 octs (1024 threads
+// would have 64 registers each: spills, and barriers of 32 warps; 32^3 solve 765
+// -> 742 us).
+template <typename T>
+constexpr int kTailThreads1 = sizeof(T) == 8 ? 512 : 1024;
 
 // Grid tail: levels [m0, split) on all CTAs, [split, last] on CTA 0.
 //
@@ -346,7 +350,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tailg(const __grid_constant__ 
 // The whole tail in one CTA: block barriers, loads through L1.  For levels
 // so small that a launch costs more than their arithmetic on one SM.
 template <typename T>
-__global__ void __launch_bounds__(kTailThreads1) k_tail1(const __grid_constant__ TailPlan plan) {
+__global__ void __launch_bounds__(kTailThreads1<T>) k_tail1(const __grid_constant__ TailPlan plan) {
   BlockSync sync;
   const FlatMap fm{(int64_t)threadIdx.x, (int64_t)blockDim.x};
   tail_body<T, false>(plan, plan.m0, fm, sync);
@@ -418,7 +422,7 @@ void tail_vcycle(cmg_level *L, int m0, const cmg_solve_params *p, const bool *ze
   LaunchScope ls(L->ctx, K_COARSE, cells * (p->n_pre + p->n_post + 2) * 3.0 * sizeof(T),
                  cells * (p->n_pre + p->n_post) * 7.0);
   if (one_cta<T>(L, m0)) {
-    k_tail1<T><<<1, kTailThreads1, 0, L->ctx->stream>>>(plan);
+    k_tail1<T><<<1, kTailThreads1<T>, 0, L->ctx->stream>>>(plan);
     CMG_CUDA(cudaGetLastError());
     return;
   }
