@@ -153,153 +153,140 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
 // nearest-upsampled `in` (Ca channels on the D/2 grid) and `skip` (Cb), read
 // in place.
 //
+// The order of the sums is part of the result: the tensor cores truncate as
+// they accumulate, an error that grows with the length of a run of MMAs (up to
+// 4e-6 of a layer's gradient between runs of different lengths), and Adam's
+// first steps and the weights' rounding to bf16 turn such a difference into
+// one of 1e-4 of the next gradients.  So a layer's bricks of 4x4x4 voxels are
+// dealt out in runs of `per_run` consecutive ones, every weight is one
+// accumulator over each run (a brick's four z slices one after the other, the
+// 16 voxels of a slice in one MMA), and the runs' sums meet in FP32 additions:
+// a training step repeats the steps of earlier versions up to the order of
+// those additions (3e-7).
+//
 // What bounds it: with 16 output channels every B fragment (16 voxels x 16
 // input channels, one ldmatrix.x4) feeds only two MMAs, so the ldmatrix reads
 // of shared memory (4 clocks each) weigh as much as the MMAs.  Hence the
-// split: blockIdx.y takes one slice of 16 input channels and all 27 taps, so
-// that a brick's halo is staged once for all of them; a warp takes the 9 taps
-// of one dz and NM tiles of 16 output channels, so that its A fragment
-// (dout^T) is read once for 9 taps and its B fragments serve NM tiles; the
-// warps left over split the brick's voxels (KW ways).  Halo and dout are kept
-// as planes of 8 channels (16-byte rows): 8 consecutive voxels are 128
-// contiguous bytes, conflict-free for ldmatrix, and a tap's offset is an
-// immediate.  Two blocks per SM walk the bricks through a cp.async ring with
-// one barrier per brick (their staging and MMA phases overlap), and a block's
-// partial sums are combined in shared memory before one red.v2 per pair of
-// weights.  The bias gradient is one more MMA per A fragment, against ones.
-// Measured on GB300, 8 blocks of 64^3 (isolated launches): 16 -> 16 channels
-// at 64^3 0.350 -> 0.101 ms (290 TFLOP/s, the mma.sync rate being about 1024
-// multiply-adds per SM and clock: 0.049 ms), 96 -> 32 at 32^3 0.950 -> 0.13
-// ms; all layers of a training step 3.6 -> 0.97 ms.
-template <int COUT, int BX, int BY, int BZ>
+// split: a block takes one run, one slice of 16 input channels, NM tiles of
+// 16 output channels (2 where the layer has them) and all 27 taps, so that a
+// brick's halo is staged once for all of them; a warp takes the 9 taps of one
+// dz, so that its A fragments (dout^T) are read once for 9 taps and its B
+// fragments serve NM tiles.  Halo rows hold their 6 voxels' lower channels and then the upper
+// ones (12 x 16 bytes), dout planes of 8 channels: the 8 addresses of an
+// ldmatrix phase (two halo rows of 4 voxels, 8 voxels of dout) lie in
+// different banks, and a tap's offset is an immediate.  Several blocks per SM
+// walk their bricks through a cp.async ring with one barrier per brick, so
+// that their staging and MMA phases overlap.  The bias gradient is one more
+// MMA per A fragment, against ones, whose 16-voxel sums are added in FP32.
+// Measured on GB300: all layers of a training step on 8 blocks of 64^3 take
+// 1.08 ms (245 TFLOP/s; the mma.sync rate, about 1024 multiply-adds per SM and
+// clock, would give 0.42 ms); with a brick's halo staged once per group of taps
+// and dout fragments read once per tap, the same sums took 3.61 ms.  Bricks of
+// 8x8x4 voxels with another order of the sums: 1.03 ms.
+// A block's output channels: 16 NM.
+template <int NM>
 struct WgradGeom {
-  static constexpr int kWarps = 6, kThreads = 32 * kWarps, kBlocks = 2;  // blocks per SM
-  static constexpr int NM = COUT == 16 ? 1 : 2;       // output-channel tiles per warp
-  static constexpr int kGroups = 3 * (COUT / 16 / NM);  // (dz, tile group)
-  static constexpr int KW = kWarps / kGroups;
-  static constexpr int HX = BX + 2, HY = BY + 2, HZ = BZ + 2, kRows = HX * HY * HZ, kVox = BX * BY * BZ;
-  // plane strides: 8 lanes of a copy (8 / planes voxels x planes) hit distinct banks
-  static constexpr int kHaloPlane = (kRows * 16 + 127) / 128 * 128 + 64;
-  static constexpr int kDoutPlane = kVox * 16 + 1024 / COUT;
-  static constexpr int kStage = (2 * kHaloPlane + (COUT / 8) * kDoutPlane + 127) / 128 * 128;
-  // The tensor cores truncate as they accumulate, an error that grows with the
-  // number of MMAs in a row: with 16 output channels (the D grid: the most
-  // bricks per block) the sums move to a second set of registers, by FP32
-  // additions, every kFlush bricks.
-  static constexpr int kFlush = COUT == 16 ? 16 : 0;
-  static constexpr int kStages = COUT == 64 ? 2 : 3;  // what two blocks per SM leave room for
-  static constexpr int kChunks = kVox / 16 / KW;       // 16-voxel chunks per warp, whole z slices
-  static constexpr int kRed = 27 * 16 * COUT * 4;
-  static constexpr int kSmem = kStages * kStage > kRed ? kStages * kStage : kRed;
+  static constexpr int kThreads = 96, kCo = 16 * NM;
+  static constexpr int kBlocks = 4;  // per SM: what the accumulators leave registers for
+  static constexpr int kStages = 3;
+  static constexpr int kHalo = 216 * 32;
+  // plane stride: 8 lanes of a copy (8 / planes voxels x planes) hit distinct banks
+  static constexpr int kDoutPlane = 64 * 16 + 1024 / kCo;
+  static constexpr int kStage = kHalo + (kCo / 8) * kDoutPlane;
+  static constexpr int kSmem = kStages * kStage;
+  static constexpr int kHaloPieces = (432 + kThreads - 1) / kThreads;  // 16-byte pieces per thread
+  static constexpr int kDoutPieces = (64 * (kCo / 8) + kThreads - 1) / kThreads;
 };
 
-template <int COUT, int BX, int BY, int BZ>
-__global__ void __launch_bounds__(WgradGeom<COUT, BX, BY, BZ>::kThreads, WgradGeom<COUT, BX, BY, BZ>::kBlocks)
-    k_conv_wgrad(const bf16 *__restrict__ dout, const bf16 *__restrict__ in,
-                                                      int CIN, const bf16 *__restrict__ skip, int Cb,
-                                                      float *__restrict__ dW, float *__restrict__ db, int D,
-                                                      int nbricks) {
-  using G = WgradGeom<COUT, BX, BY, BZ>;
-  constexpr int NM = G::NM, kUnroll = NM == 1 ? G::kChunks : 1;  // one tile leaves registers to unroll
+template <int NM>
+__global__ void __launch_bounds__(WgradGeom<NM>::kThreads, WgradGeom<NM>::kBlocks)
+    k_conv_wgrad(const bf16 *__restrict__ dout, int COUT, const bf16 *__restrict__ in, int CIN,
+                 const bf16 *__restrict__ skip, int Cb, float *__restrict__ dW, float *__restrict__ db, int D,
+                 int nbricks, int per_run) {
+  using G = WgradGeom<NM>;
+  constexpr int C8 = G::kCo / 8, kUnroll = NM == 1 ? 4 : 1;  // one tile leaves registers to unroll
   extern __shared__ __align__(16) uint8_t smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int group = warp % G::kGroups, kw = warp / G::kGroups;
-  const int dz = group % 3, mb0 = (group / 3) * NM;
-  const int nbx = D / BX, nby = D / BY, per = nbx * nby * (D / BZ);
+  const int lane = threadIdx.x & 31, dz = threadIdx.x >> 5, co_first = blockIdx.z * G::kCo;
+  const int first = blockIdx.x * per_run, last = min(first + per_run, nbricks);
+  const int nb = D >> 2;
   // this block's slice of 16 input channels
   const int Ca = CIN - Cb, c_first = blockIdx.y * 16;
   const bool two = skip != nullptr, up = two && c_first < Ca;
-  const bf16 *src = (two && !up) ? skip : in;
   const int cstride = up ? Ca : (two ? Cb : CIN), cbase = (two && !up) ? c_first - Ca : c_first;
+  const bf16 *src = ((two && !up) ? skip : in) + cbase;
   const int Dg = up ? D >> 1 : D, sh = up ? 1 : 0;
+  const uint32_t base = smem_u32(smem);
 
-  auto stage = [&](int bi, int buf) {
-    const int s = bi / per, brick = bi % per;
-    const int x0 = (brick % nbx) * BX, y0 = ((brick / nbx) % nby) * BY, z0 = (brick / (nbx * nby)) * BZ;
-    const uint32_t halo = smem_u32(smem + buf * G::kStage), dt = halo + 2 * G::kHaloPlane;
-    const bf16 *ss = src + (int64_t)s * Dg * Dg * Dg * cstride + cbase;
-    // a warp copies rows of halo voxels of one z, lane = (x, channel half)
-    const int hx = lane >> 1, half = lane & 1;
-    const bf16 *sx = ss + (int64_t)(wrap(x0 + hx - 1, D) >> sh) * cstride + half * 8;
-    const uint32_t dst = halo + half * G::kHaloPlane + hx * 16;
-    if (hx < G::HX) {
-      for (int hz = warp; hz < G::HZ; hz += G::kWarps) {
-        const bf16 *sz = sx + (int64_t)(wrap(z0 + hz - 1, D) >> sh) * Dg * Dg * cstride;
+  // the brick staged next
+  int bx = first % nb, by = (first / nb) % nb, bz = (first / (nb * nb)) % nb, smp = first / (nb * nb * nb);
+  auto stage = [&](int buf) {
+    const uint32_t halo = base + buf * G::kStage, dt = halo + G::kHalo;
+    const bf16 *ss = src + (int64_t)smp * Dg * Dg * Dg * cstride;
+    const int x0 = bx * 4, y0 = by * 4, z0 = bz * 4;
+    // 16-byte pieces in the order of the rows in shared memory: voxel (hz, hy,
+    // hx) and channel half
 #pragma unroll
-        for (int hy = 0; hy < G::HY; ++hy)
-          cp_async16(dst + (hz * G::HY + hy) * (G::HX * 16), sz + (wrap(y0 + hy - 1, D) >> sh) * Dg * cstride);
-      }
+    for (int k = 0; k < G::kHaloPieces; ++k) {
+      const int p = threadIdx.x + k * G::kThreads;
+      const int hz = p / 72, hy = (p / 12) % 6, half = (p / 6) & 1, hx = p % 6;
+      const int z = wrap(z0 + hz - 1, D) >> sh, y = wrap(y0 + hy - 1, D) >> sh, x = wrap(x0 + hx - 1, D) >> sh;
+      if (p < 432) cp_async16(halo + p * 16, ss + ((int64_t)(z * Dg + y) * Dg + x) * cstride + half * 8);
     }
-    // dout: 32 consecutive 16-byte pieces of a row of BX voxels per warp
-    const bf16 *ds = dout + ((((int64_t)s * D + z0) * D + y0) * D + x0) * COUT;
-    constexpr int kC8 = COUT / 8, kRow = BX * kC8;  // pieces per voxel, per row
-    for (int p = threadIdx.x; p < G::kVox * kC8; p += G::kThreads) {
-      const int r = p / kRow, i = p % kRow;
-      cp_async16(dt + (i % kC8) * G::kDoutPlane + (r * BX + i / kC8) * 16, ds + ((r / BY) * D + r % BY) * D * COUT + i * 8);
+    const bf16 *ds = dout + ((((int64_t)smp * D + z0) * D + y0) * D + x0) * COUT + co_first;
+#pragma unroll
+    for (int k = 0; k < G::kDoutPieces; ++k) {
+      const int p = threadIdx.x + k * G::kThreads, v = p / C8, c8 = p % C8;
+      if (p < 64 * C8)
+        cp_async16(dt + c8 * G::kDoutPlane + v * 16, ds + (((v >> 4) * D + ((v >> 2) & 3)) * D + (v & 3)) * COUT + c8 * 8);
+    }
+    if (++bx == nb) {
+      bx = 0;
+      if (++by == nb) {
+        by = 0;
+        if (++bz == nb) {
+          bz = 0;
+          ++smp;
+        }
+      }
     }
   };
 
-  float acc[9][NM][2][4], accb[NM][4];
-  constexpr int kTot = G::kFlush ? 9 * NM * 8 + NM * 4 : 1;
-  float tot[kTot];
-#pragma unroll
-  for (int k = 0; k < kTot; ++k) tot[k] = 0.f;
-  auto flush = [&]() {
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-#pragma unroll
-      for (int k = 0; k < 72; ++k) {
-        float &x = acc[k / 8][m][(k / 4) % 2][k % 4];
-        tot[m * 72 + k] += x;
-        x = 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        tot[NM * 72 + m * 4 + k] += accb[m][k];
-        accb[m][k] = 0.f;
-      }
-    }
-  };
+  float acc[9][NM][2][4], sum[NM][2];
 #pragma unroll
   for (int m = 0; m < NM; ++m) {
 #pragma unroll
     for (int t = 0; t < 9; ++t)
 #pragma unroll
       for (int h = 0; h < 2; ++h) acc[t][m][h][0] = acc[t][m][h][1] = acc[t][m][h][2] = acc[t][m][h][3] = 0.f;
-    accb[m][0] = accb[m][1] = accb[m][2] = accb[m][3] = 0.f;
+    sum[m][0] = sum[m][1] = 0.f;
   }
   const bool bias = blockIdx.y == 0 && dz == 0;
   const int bk = (lane & 7) + ((lane >> 3) & 1) * 8, bhalf = (lane >> 4) & 1;  // B rows: voxel bk, channel half
   const int ak = (lane & 7) + ((lane >> 4) & 1) * 8, ahalf = (lane >> 3) & 1;  // A rows
-  const uint32_t lane_a = ahalf * G::kDoutPlane + (kw * G::kChunks * 16 + ak) * 16;
-  const uint32_t lane_b = bhalf * G::kHaloPlane +
-                          ((kw * G::kChunks * 16 / (BX * BY) + dz) * (G::HX * G::HY) + (bk / BX) * G::HX + bk % BX) * 16;
-  int buf = 0, since = 0;
+  const uint32_t lane_a = G::kHalo + ahalf * G::kDoutPlane + ak * 16;
+  const uint32_t lane_b = ((dz * 6 + (bk >> 2)) * 12 + bhalf * 6 + (bk & 3)) * 16;
+  int buf = 0;
 #pragma unroll
   for (int k = 0; k < G::kStages - 1; ++k) {
-    if (blockIdx.x + k * (int)gridDim.x < nbricks) stage(blockIdx.x + k * gridDim.x, k);
+    if (first + k < last) stage(k);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  for (int bi = blockIdx.x; bi < nbricks; bi += gridDim.x, buf = buf + 1 == G::kStages ? 0 : buf + 1) {
-    if (G::kStages == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
-    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+  for (int bi = first; bi < last; ++bi, buf = buf + 1 == G::kStages ? 0 : buf + 1) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(G::kStages - 2) : "memory");
     __syncthreads();  // this brick has landed, and the buffer filled next was read a brick ago
-    const int nx = bi + (G::kStages - 1) * (int)gridDim.x;
-    if (nx < nbricks) stage(nx, buf == 0 ? G::kStages - 1 : buf - 1);
+    if (bi + G::kStages - 1 < last) stage(buf == 0 ? G::kStages - 1 : buf - 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const uint32_t halo = smem_u32(smem + buf * G::kStage), dt = halo + 2 * G::kHaloPlane;
+    const uint32_t at = base + buf * G::kStage;
 #pragma unroll(kUnroll)
-    for (int i = 0; i < G::kChunks; ++i) {
+    for (int i = 0; i < 4; ++i) {  // the brick's z slices
       uint32_t a[NM][4];
 #pragma unroll
       for (int m = 0; m < NM; ++m)
-        ldsm_x4_t(dt + lane_a + 2 * (mb0 + m) * G::kDoutPlane + i * 256, a[m][0], a[m][1], a[m][2], a[m][3]);
-      const uint32_t hb =
-          halo + lane_b + ((i * 16 / (BX * BY)) * (G::HX * G::HY) + (i * 16 % (BX * BY)) / BX * G::HX) * 16;
+        ldsm_x4_t(at + lane_a + 2 * m * G::kDoutPlane + i * 256, a[m][0], a[m][1], a[m][2], a[m][3]);
 #pragma unroll
       for (int t = 0; t < 9; ++t) {
         uint32_t b0, b1, b2, b3;
-        ldsm_x4_t(hb + ((t / 3) * G::HX + t % 3) * 16, b0, b1, b2, b3);
+        ldsm_x4_t(at + lane_b + ((i * 6 + t / 3) * 12 + t % 3) * 16, b0, b1, b2, b3);
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
           mma16816(acc[t][m][0], a[m][0], a[m][1], a[m][2], a[m][3], b0, b1);
@@ -309,67 +296,32 @@ __global__ void __launch_bounds__(WgradGeom<COUT, BX, BY, BZ>::kThreads, WgradGe
       if (bias) {
         constexpr uint32_t kOnes = 0x3F803F80u;  // bf16 1, 1
 #pragma unroll
-        for (int m = 0; m < NM; ++m) mma16816(accb[m], a[m][0], a[m][1], a[m][2], a[m][3], kOnes, kOnes);
-      }
-    }
-    if constexpr (G::kFlush > 0) {
-      if (++since == G::kFlush) {
-        flush();
-        since = 0;
+        for (int m = 0; m < NM; ++m) {
+          float c[4] = {0.f, 0.f, 0.f, 0.f};
+          mma16816(c, a[m][0], a[m][1], a[m][2], a[m][3], kOnes, kOnes);
+          sum[m][0] += c[0];
+          sum[m][1] += c[2];
+        }
       }
     }
   }
-  if constexpr (G::kFlush > 0) {
-    flush();
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-#pragma unroll
-      for (int k = 0; k < 72; ++k) acc[k / 8][m][(k / 4) % 2][k % 4] = tot[m * 72 + k];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) accb[m][k] = tot[NM * 72 + m * 4 + k];
-    }
-  }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
-  // the KW partial sums of each (tap, co, ci), then one red.v2 per pair of ci
-  float *red = reinterpret_cast<float *>(smem);  // [27][COUT][16]
+  // one red.v2 per pair of ci
   const int g = lane >> 2, q = lane & 3;
-#pragma unroll 1
-  for (int w = 0; w < G::KW; ++w) {
-    if (kw == w) {
+#pragma unroll
+  for (int m = 0; m < NM; ++m)
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const int co = co_first + m * 16 + g + 8 * hh;
+      float *dst = dW + ((int64_t)co * 27 + dz * 9) * CIN + c_first + 2 * q;
 #pragma unroll
       for (int t = 0; t < 9; ++t)
 #pragma unroll
-        for (int m = 0; m < NM; ++m)
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              float2 *r = reinterpret_cast<float2 *>(red + ((dz * 9 + t) * COUT + (mb0 + m) * 16 + g + 8 * hh) * 16 +
-                                                     8 * h + 2 * q);
-              float2 x = make_float2(acc[t][m][h][2 * hh], acc[t][m][h][2 * hh + 1]);
-              if (w > 0) {
-                const float2 o = *r;
-                x.x += o.x;
-                x.y += o.y;
-              }
-              *r = x;
-            }
+        for (int h = 0; h < 2; ++h)
+          asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dst + t * CIN + 8 * h),
+                       "f"(acc[t][m][h][2 * hh]), "f"(acc[t][m][h][2 * hh + 1])
+                       : "memory");
+      if (bias && q == 0) atomicAdd(db + co, sum[m][hh]);
     }
-    __syncthreads();
-  }
-  for (int p = threadIdx.x; p < 27 * COUT * 8; p += G::kThreads) {
-    const int j = p & 7, co = (p >> 3) % COUT, t = p / (8 * COUT);
-    const float2 x = reinterpret_cast<const float2 *>(red)[p];
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dW + ((int64_t)co * 27 + t) * CIN + c_first + 2 * j),
-                 "f"(x.x), "f"(x.y)
-                 : "memory");
-  }
-  if (bias && q == 0)
-#pragma unroll
-    for (int m = 0; m < NM; ++m)
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh) atomicAdd(db + (mb0 + m) * 16 + g + 8 * hh, accb[m][2 * hh]);
 }
 
 // ---- per-sample input statistics and the network input
@@ -487,7 +439,8 @@ __global__ void k_head(const bf16 *__restrict__ d0, const float *__restrict__ hw
 // loss = mean (delta - target)^2, target = (phi_next - phi_prev) / rms;
 // ddelta = 2 (delta - target) / (B V); dact = bf16(ddelta w) where d0 > 0,
 // else 0 (the ReLU derivative); head grads.  One voxel (32 bytes of d0 and
-// dact) per thread and step; the 18 block sums are formed by few blocks.
+// dact) per thread and step.  The grid is part of the head gradients' rounding
+// (see k_conv_wgrad): up to 4096 blocks, whose FP32 sums are added up.
 __global__ void __launch_bounds__(256) k_head_grad(const bf16 *__restrict__ d0, const float *__restrict__ hw,
                                                   const float *__restrict__ delta, const float *__restrict__ phi_prev,
                                                   const float *__restrict__ phi_next, const float *__restrict__ norm,
@@ -853,39 +806,32 @@ void conv(cmg_unet *U, int l, const bf16 *in, int K, const float *bias, const bf
 #undef CMG_CONV
 }
 
-template <int COUT, int BX, int BY, int BZ>
-void wgrad_launch(cmg_unet *U, const bf16 *dout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW, float *db,
-                  int D, int B) {
-  using G = WgradGeom<COUT, BX, BY, BZ>;
+template <int NM>
+void wgrad_launch(cmg_unet *U, const bf16 *dout, int Cout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW,
+                  float *db, int D, int B) {
+  using G = WgradGeom<NM>;
   static int attr_dev = -1;
   if (attr_dev != U->ctx->device) {
-    CMG_CUDA(cudaFuncSetAttribute(k_conv_wgrad<COUT, BX, BY, BZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  G::kSmem));
+    CMG_CUDA(cudaFuncSetAttribute(k_conv_wgrad<NM>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem));
     attr_dev = U->ctx->device;
   }
-  const int nbricks = B * (D / BX) * (D / BY) * (D / BZ), slices = Cin / 16;
-  const int blocks = std::max(1, std::min(nbricks, G::kBlocks * U->ctx->num_sms / slices));
-  LaunchScope ls(U->ctx, K_CONV_WGRAD, 0.0, 2.0 * 27 * COUT * Cin * (double)D * D * D * B);
-  k_conv_wgrad<COUT, BX, BY, BZ><<<dim3(blocks, slices), G::kThreads, G::kSmem, U->ctx->stream>>>(
-      dout, in, Cin, skip, Cb, dW, db, D, nbricks);
+  // Runs of bricks (k_conv_wgrad): about 4 per SM, a third or a ninth as many
+  // where the layer has more than 3 or 8 tiles of 16 x 16 channels.
+  const int nbricks = B * (D / 4) * (D / 4) * (D / 4), slices = Cin / 16, tiles = slices * (Cout / 16);
+  const int most = std::max(1, std::min(nbricks, 4 * U->ctx->num_sms / (tiles <= 3 ? 1 : tiles <= 8 ? 3 : 9)));
+  const int per_run = (nbricks + most - 1) / most, runs = (nbricks + per_run - 1) / per_run;
+  LaunchScope ls(U->ctx, K_CONV_WGRAD, 0.0, 2.0 * 27 * Cout * Cin * (double)D * D * D * B);
+  k_conv_wgrad<NM><<<dim3(runs, slices, Cout / G::kCo), G::kThreads, G::kSmem, U->ctx->stream>>>(
+      dout, Cout, in, Cin, skip, Cb, dW, db, D, nbricks, per_run);
   CMG_CUDA(cudaGetLastError());
 }
 
-// Weight and bias gradients; bricks of 8 x 8 x 4 voxels, 4 x 4 x 4 on grids
-// that 8 does not divide.  skip: see k_conv_wgrad.
+// Weight and bias gradients; skip: see k_conv_wgrad.
 void wgrad(cmg_unet *U, const bf16 *dout, int Cout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW,
            float *db, int D, int B) {
-#define CMG_WG(CO)                                                                        \
-  if (Cout == CO) {                                                                       \
-    if (D % 8 == 0) wgrad_launch<CO, 8, 8, 4>(U, dout, in, Cin, skip, Cb, dW, db, D, B);  \
-    else wgrad_launch<CO, 4, 4, 4>(U, dout, in, Cin, skip, Cb, dW, db, D, B);             \
-    return;                                                                               \
-  }
-  CMG_WG(16)
-  CMG_WG(32)
-  CMG_WG(64)
-#undef CMG_WG
-  throw Error(CMG_ERR_INVALID_ARG, "unsupported channel count");
+  if (Cin % 16 || (Cout != 16 && Cout % 32)) throw Error(CMG_ERR_INVALID_ARG, "unsupported channel count");
+  if (Cout == 16) wgrad_launch<1>(U, dout, Cout, in, Cin, skip, Cb, dW, db, D, B);
+  else wgrad_launch<2>(U, dout, Cout, in, Cin, skip, Cb, dW, db, D, B);
 }
 
 // After a synchronisation: a bounded wait that expired in a tcgen05
@@ -1008,7 +954,7 @@ void backward(cmg_unet *U, int B, const Fields &F) {
   CMG_CUDA(cudaMemsetAsync(U->grads, 0, sizeof(float) * U->np, s));
   CMG_CUDA(cudaMemsetAsync(U->loss, 0, sizeof(double), s));
   float *ghw = U->grads + layer_offset(10);
-  k_head_grad<<<std::min<int64_t>(gsz(B * V0), 4 * U->ctx->num_sms), 256, 0, s>>>(
+  k_head_grad<<<gsz(B * V0), 256, 0, s>>>(
       U->a[9], U->params + layer_offset(10), F.delta, F.base, F.next, U->norm, V0, B, U->g0, ghw, ghw + 16,
       U->loss);
   CMG_CUDA(cudaGetLastError());
