@@ -373,7 +373,14 @@ int cmg_batch_autotune(cmg_batch *batch, const cmg_solve_params *params, cmg_bat
  * vector (per layer [Cout][27][Cin] weights then biases; head 16 + 1);
  * convolutions run on BF16 weights and BF16 activations with FP32
  * accumulation (tensor cores), the head and the optimiser in FP32.
- * Fields are dense [batch][D][D][D] (z, y, x) FP32 arrays in `mem`. */
+ * Fields are dense [batch][D][D][D] (z, y, x) FP32 arrays in `mem`.  A call on
+ * device arrays is queued on the context's stream: its kernels read the inputs
+ * and write the outputs in place, up to the last one of the call, so other
+ * streams must leave the arrays alone until that work is done.  Outputs may
+ * overlap inputs and each other (as if the inputs were copied first and pred,
+ * then delta, written last; such calls take extra copies).  Host arrays in a
+ * call on device memory (or the reverse) are copied, and the call then waits
+ * for its copies. */
 typedef struct cmg_unet cmg_unet;
 /* grid_dim: multiple of 16; max_batch: samples per call. */
 int cmg_unet_create(cmg_ctx *ctx, int grid_dim, int max_batch, cmg_unet **out);

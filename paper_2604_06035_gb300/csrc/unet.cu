@@ -991,17 +991,57 @@ void backward(cmg_unet *U, int B, const Fields &F) {
   CMG_CUDA(cudaGetLastError());
 }
 
-void copy_in(cmg_unet *U, float *dst, const float *src, int64_t n, int mem) {
-  CMG_CUDA(cudaMemcpyAsync(dst, src, sizeof(float) * n,
-                           mem == CMG_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, U->ctx->stream));
+// The kind is left to the runtime: one memory flag stands for all arrays of a
+// call, and an array of the other kind is copied all the same.
+void copy_async(cmg_unet *U, void *dst, const void *src, int64_t bytes) {
+  CMG_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, U->ctx->stream));
 }
 
-// An input field on the device: src itself, or buf with a copy of host memory.
-const float *field_in(cmg_unet *U, float *buf, const float *src, int64_t n, int mem) {
-  if (mem != CMG_MEM_HOST) return src;
-  copy_in(U, buf, src, n, mem);
-  return buf;
-}
+// The fields of a device-memory call are read and written in place where that
+// gives what copies of the inputs at the start and of the outputs at the end
+// give; else they go through the network's buffers.
+struct FieldArgs {
+  cmg_unet *U;
+  int64_t n;          // values per field
+  bool host;          // a host-memory call
+  bool wait = false;  // host memory is copied: the call waits for it
+
+  static cudaPointerAttributes where(const void *p) {
+    cudaPointerAttributes a = {};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+      cudaGetLastError();
+      a.type = cudaMemoryTypeUnregistered;
+    }
+    return a;
+  }
+  // memory that the kernels can take as it is: the context's GPU's own (host
+  // memory in a call marked as device memory is not, nor another GPU's)
+  bool resident(const void *p) const {
+    if (host) return false;
+    const cudaPointerAttributes a = where(p);
+    return a.type == cudaMemoryTypeDevice && a.device == U->ctx->device;
+  }
+  void copy(float *dst, const float *src, const void *callers) {
+    copy_async(U, dst, src, sizeof(float) * n);
+    const cudaMemoryType t = where(callers).type;
+    wait = wait || t == cudaMemoryTypeUnregistered || t == cudaMemoryTypeHost;
+  }
+  const float *in(float *buf, const float *src) {
+    if (resident(src)) return src;
+    copy(buf, src, src);
+    return buf;
+  }
+  bool overlap(const float *a, const float *b) const { return a && b && a < b + n && b < a + n; }
+  // Where the kernels write an output.  The last one reads the base field and
+  // writes both outputs, voxel by voxel, so none of the three may overlap.
+  float *out(float *buf, float *dst, const float *base, const float *other) const {
+    if (!dst) return nullptr;
+    return resident(dst) && !overlap(dst, base) && !overlap(dst, other) ? dst : buf;
+  }
+  void deliver(float *dst, const float *from) {
+    if (dst && dst != from) copy(dst, from, dst);
+  }
+};
 
 }  // namespace
 }  // namespace cmg
@@ -1110,8 +1150,9 @@ int cmg_unet_set_params(cmg_unet *U, const float *params, cmg_mem mem) {
   return unet_guard([&] {
     if (!U || !params) return (int)CMG_ERR_INVALID_ARG;
     cudaSetDevice(U->ctx->device);
-    cmg::copy_in(U, U->params, params, U->np, mem);
     cudaStream_t s = U->ctx->stream;
+    CMG_CUDA(cudaMemcpyAsync(U->params, params, sizeof(float) * U->np,
+                             mem == CMG_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
     CMG_CUDA(cudaMemsetAsync(U->m, 0, sizeof(float) * U->np, s));
     CMG_CUDA(cudaMemsetAsync(U->v, 0, sizeof(float) * U->np, s));
     CMG_CUDA(cudaMemsetAsync(U->clip, 0, sizeof(double) * 8, s));
@@ -1159,20 +1200,18 @@ int cmg_unet_forward(cmg_unet *U, const float *rho, const float *field, const fl
     cudaSetDevice(U->ctx->device);
     const int64_t n = (int64_t)batch * U->D * U->D * U->D;
     cudaStream_t s = U->ctx->stream;
-    const bool host = mem == CMG_MEM_HOST;
+    cmg::FieldArgs A = {U, n, mem == CMG_MEM_HOST};
     cmg::Fields F = {};
-    F.rho = cmg::field_in(U, U->in_rho, rho, n, mem);
-    F.phi = cmg::field_in(U, U->in_phi, field, n, mem);
-    F.base = base ? cmg::field_in(U, U->in_base, base, n, mem) : F.phi;
-    F.pred = !phi_pred ? nullptr : host ? U->out_phi : phi_pred;
-    F.delta = !delta ? nullptr : host ? U->delta : delta;
+    F.rho = A.in(U->in_rho, rho);
+    F.phi = A.in(U->in_phi, field);
+    F.base = base ? A.in(U->in_base, base) : F.phi;
+    F.pred = A.out(U->out_phi, phi_pred, F.base, delta);
+    F.delta = A.out(U->delta, delta, F.base, phi_pred);
     cmg::forward(U, batch, F, false);
-    if (host) {
-      if (phi_pred) CMG_CUDA(cudaMemcpyAsync(phi_pred, U->out_phi, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
-      if (delta) CMG_CUDA(cudaMemcpyAsync(delta, U->delta, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
-      CMG_CUDA(cudaStreamSynchronize(s));
-      cmg::check_status(U);
-    }
+    A.deliver(phi_pred, F.pred);
+    A.deliver(delta, F.delta);
+    if (A.host || A.wait) CMG_CUDA(cudaStreamSynchronize(s));
+    if (A.host) cmg::check_status(U);
     return (int)CMG_OK;
   });
 }
@@ -1184,11 +1223,12 @@ int cmg_unet_gradients(cmg_unet *U, const float *rho, const float *field, const 
     cudaSetDevice(U->ctx->device);
     const int64_t n = (int64_t)batch * U->D * U->D * U->D;
     cudaStream_t s = U->ctx->stream;
+    cmg::FieldArgs A = {U, n, mem == CMG_MEM_HOST};
     cmg::Fields F = {};
-    F.rho = cmg::field_in(U, U->in_rho, rho, n, mem);
-    F.phi = cmg::field_in(U, U->in_phi, field, n, mem);
-    F.base = base ? cmg::field_in(U, U->in_base, base, n, mem) : F.phi;
-    F.next = cmg::field_in(U, U->in_next, target, n, mem);
+    F.rho = A.in(U->in_rho, rho);
+    F.phi = A.in(U->in_phi, field);
+    F.base = base ? A.in(U->in_base, base) : F.phi;
+    F.next = A.in(U->in_next, target);
     F.delta = U->delta;
     cmg::forward(U, batch, F, true);
     cmg::backward(U, batch, F);
@@ -1197,7 +1237,8 @@ int cmg_unet_gradients(cmg_unet *U, const float *rho, const float *field, const 
     if (loss) {
       CMG_CUDA(cudaMemcpyAsync(loss, U->loss, sizeof(double), k, s));
     }
-    if (mem == CMG_MEM_HOST || loss) {
+    if (A.wait && !A.host && !loss) CMG_CUDA(cudaStreamSynchronize(s));
+    if (A.host || loss) {
       CMG_CUDA(cudaStreamSynchronize(s));
       cmg::check_status(U);
     }
