@@ -180,6 +180,9 @@ int cmg_level_build128(cmg_ctx *ctx, int level, int nx, int periodic_mask, const
                        int64_t n_octs, cmg_mem mem, cmg_level *parent, cmg_level **out);
 /* 64 or 128. */
 int cmg_level_key_bits(const cmg_level *lvl, int *bits);
+/* Waits for the level's work and frees it.  While other levels of the context
+ * are alive, the context keeps up to 512 MiB of the freed device memory for the
+ * levels it builds next; the last level to be destroyed gives all of it back. */
 int cmg_level_destroy(cmg_level *lvl);
 int cmg_level_n_octs(const cmg_level *lvl, int64_t *n_octs);
 /* Hash capacity (power of two) of the level's table. */

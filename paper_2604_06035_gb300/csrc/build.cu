@@ -77,6 +77,10 @@ LevelMemory::~LevelMemory() {
   if (pool) cudaMemPoolDestroy(pool);
 }
 
+void LevelMemory::trim() {
+  if (cudaMemPoolTrimTo(pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
 void *LevelMemory::take_pinned() {
   {
     std::lock_guard<std::mutex> lock(m);

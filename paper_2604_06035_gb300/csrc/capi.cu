@@ -339,6 +339,14 @@ int cmg_morton_decode128(cmg_ctx *ctx, const uint64_t *keys, int64_t n, uint64_t
 
 namespace {
 
+// The level's memory goes to the context's pool, and with the last level of a
+// context the pool's to the GPU.
+void release_level(cmg_level *L) {
+  L->mem.release();
+  if (L->memory.use_count() <= 2) L->memory->trim();  // this level and, at most, the context
+  delete L;
+}
+
 int level_build(cmg_ctx *ctx, int level, int nx, int periodic_mask, const void *keys, int64_t n_octs, cmg_mem mem,
                 cmg_level *parent, cmg_level **out, int key_bits) {
   return guard([&] {
@@ -382,8 +390,7 @@ int level_build(cmg_ctx *ctx, int level, int nx, int periodic_mask, const void *
       CMG_CUDA(cudaStreamSynchronize(ctx->stream));
     } catch (...) {
       cudaStreamSynchronize(ctx->stream);
-      L->mem.release();
-      delete L;
+      release_level(L);
       throw;
     }
     *out = L;
@@ -421,8 +428,7 @@ int cmg_level_destroy(cmg_level *lvl) {
   if (lvl->h_ctrl) lvl->memory->give_pinned(lvl->h_ctrl);
   if (lvl->ev_start) cudaEventDestroy(lvl->ev_start);
   if (lvl->ev_end) cudaEventDestroy(lvl->ev_end);
-  lvl->mem.release();
-  delete lvl;
+  release_level(lvl);
   if (prev >= 0) cudaSetDevice(prev);
   return CMG_OK;
 }

@@ -210,7 +210,8 @@ struct MgLev {
 // freed memory, and a few pinned blocks for solve control words.  Rebuilding
 // and destroying a 178k-oct level took 1.45 + 0.93 ms without it.  Shared by
 // the context and its levels (a level may outlive its context); the last of
-// them gives everything back.
+// them gives everything back, and the last level to be destroyed all of the
+// pool's memory.
 struct LevelMemory {
   static constexpr uint64_t kKept = uint64_t(512) << 20;
   static constexpr size_t kPinnedBytes = 4096, kPinnedKept = 8;
@@ -218,6 +219,7 @@ struct LevelMemory {
   ~LevelMemory();
   void *take_pinned();
   void give_pinned(void *p);
+  void trim();  // gives back the freed memory that the pool holds
   cudaMemPool_t pool = nullptr;
 
  private:
