@@ -428,6 +428,15 @@ int cmg_unet_set_grad_clip(cmg_unet *net, float k);
  * (before capping), the running mean, steps seen and steps capped; any
  * pointer may be NULL. */
 int cmg_unet_grad_clip_stats(cmg_unet *net, double *last_norm, double *mean_norm, int64_t *steps, int64_t *clipped);
+/* Tests: the weight and bias gradients of one convolution, as the training
+ * step's kernel forms them.  dout [batch][D^3][cout] (cout 16, 32 or 64), in
+ * [batch][D^3][cin] (cin a multiple of 16 up to 96) as bf16 bit patterns;
+ * with skip [batch][D^3][skip_channels], in holds the other cin -
+ * skip_channels channels on the grid of D/2 and is upsampled.  dw
+ * [cout][27][cin] and db [cout] are replaced.  D a multiple of 4; 16-byte
+ * aligned device memory; queued on the context's stream. */
+int cmg_debug_conv_wgrad(cmg_ctx *ctx, const uint16_t *dout, int cout, const uint16_t *in, int cin,
+                         const uint16_t *skip, int skip_channels, int grid_dim, int batch, float *dw, float *db);
 /* Device copy between a dense [D][D][D] (z, y, x) FP64 field and the oct-major
  * [n][8] field of the full periodic level whose octs are listed x fastest
  * (to_octs = 1: dense -> octs; 0: octs -> dense).  Both device pointers. */

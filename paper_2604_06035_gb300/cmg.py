@@ -146,6 +146,7 @@ _SIGS = {
     "cmg_unet_adam_step": (_I, [_P, C.c_float, C.c_float, C.c_float, C.c_float]),
     "cmg_unet_set_grad_clip": (_I, [_P, C.c_float]),
     "cmg_unet_grad_clip_stats": (_I, [_P, C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(_I64), C.POINTER(_I64)]),
+    "cmg_debug_conv_wgrad": (_I, [_P, _P, _I, _P, _I, _P, _I, _I, _I, _P, _P]),
     "cmg_dense_octs": (_I, [_P, _P, _I, _P, _I]),
 }
 
@@ -835,6 +836,30 @@ def cmg_unet_grad_clip_stats(net):
     _check(lib().cmg_unet_grad_clip_stats(net.h, C.byref(last), C.byref(mean), C.byref(steps), C.byref(clipped)),
            "cmg_unet_grad_clip_stats")
     return {"last_norm": last.value, "mean_norm": mean.value, "steps": steps.value, "clipped": clipped.value}
+
+
+def cmg_debug_conv_wgrad(ctx, dout, inp, skip=None):
+    """Tests: (dw [cout, 27, cin], db [cout]) of one convolution from bfloat16
+    CUDA tensors dout [B, D, D, D, cout] and inp [B, D, D, D, cin]; with skip
+    [B, D, D, D, cb], inp is the upsampled part on the grid of D/2."""
+    import torch
+    B, D, cout = dout.shape[0], dout.shape[1], dout.shape[-1]
+    cb = 0 if skip is None else skip.shape[-1]
+    cin = inp.shape[-1] + cb
+    half = 1 if skip is None else 2
+    for t, shape in ((dout, (B, D, D, D, cout)), (inp, (B,) + (D // half,) * 3 + (cin - cb,)), (skip, (B, D, D, D, cb))):
+        if t is None:
+            continue
+        if t.dtype != torch.bfloat16 or not t.is_cuda or not t.is_contiguous() or t.data_ptr() % 16:
+            raise TypeError("cmg_debug_conv_wgrad takes contiguous bfloat16 CUDA tensors on 16-byte boundaries")
+        if tuple(t.shape) != shape:
+            raise ValueError("cmg_debug_conv_wgrad: an array has shape %s, not %s" % (tuple(t.shape), shape))
+    dw = torch.empty((cout, 27, cin), dtype=torch.float32, device=dout.device)
+    db = torch.empty(cout, dtype=torch.float32, device=dout.device)
+    _check(lib().cmg_debug_conv_wgrad(ctx, dout.data_ptr(), cout, inp.data_ptr(), cin,
+                                      None if skip is None else skip.data_ptr(), cb, D, B, dw.data_ptr(),
+                                      db.data_ptr()), "cmg_debug_conv_wgrad")
+    return dw, db
 
 
 def cmg_dense_octs(ctx, src, grid_dim, dst, to_octs):

@@ -807,31 +807,27 @@ void conv(cmg_unet *U, int l, const bf16 *in, int K, const float *bias, const bf
 }
 
 template <int NM>
-void wgrad_launch(cmg_unet *U, const bf16 *dout, int Cout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW,
+void wgrad_launch(cmg_ctx *ctx, const bf16 *dout, int Cout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW,
                   float *db, int D, int B) {
   using G = WgradGeom<NM>;
-  static int attr_dev = -1;
-  if (attr_dev != U->ctx->device) {
-    CMG_CUDA(cudaFuncSetAttribute(k_conv_wgrad<NM>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem));
-    attr_dev = U->ctx->device;
-  }
+  static_assert(G::kSmem <= 48 * 1024, "more needs an attribute");
   // Runs of bricks (k_conv_wgrad): about 4 per SM, a third or a ninth as many
   // where the layer has more than 3 or 8 tiles of 16 x 16 channels.
   const int nbricks = B * (D / 4) * (D / 4) * (D / 4), slices = Cin / 16, tiles = slices * (Cout / 16);
-  const int most = std::max(1, std::min(nbricks, 4 * U->ctx->num_sms / (tiles <= 3 ? 1 : tiles <= 8 ? 3 : 9)));
+  const int most = std::max(1, std::min(nbricks, 4 * ctx->num_sms / (tiles <= 3 ? 1 : tiles <= 8 ? 3 : 9)));
   const int per_run = (nbricks + most - 1) / most, runs = (nbricks + per_run - 1) / per_run;
-  LaunchScope ls(U->ctx, K_CONV_WGRAD, 0.0, 2.0 * 27 * Cout * Cin * (double)D * D * D * B);
-  k_conv_wgrad<NM><<<dim3(runs, slices, Cout / G::kCo), G::kThreads, G::kSmem, U->ctx->stream>>>(
+  LaunchScope ls(ctx, K_CONV_WGRAD, 0.0, 2.0 * 27 * Cout * Cin * (double)D * D * D * B);
+  k_conv_wgrad<NM><<<dim3(runs, slices, Cout / G::kCo), G::kThreads, G::kSmem, ctx->stream>>>(
       dout, Cout, in, Cin, skip, Cb, dW, db, D, nbricks, per_run);
   CMG_CUDA(cudaGetLastError());
 }
 
 // Weight and bias gradients; skip: see k_conv_wgrad.
-void wgrad(cmg_unet *U, const bf16 *dout, int Cout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW,
+void wgrad(cmg_ctx *ctx, const bf16 *dout, int Cout, const bf16 *in, int Cin, const bf16 *skip, int Cb, float *dW,
            float *db, int D, int B) {
   if (Cin % 16 || (Cout != 16 && Cout % 32)) throw Error(CMG_ERR_INVALID_ARG, "unsupported channel count");
-  if (Cout == 16) wgrad_launch<1>(U, dout, Cout, in, Cin, skip, Cb, dW, db, D, B);
-  else wgrad_launch<2>(U, dout, Cout, in, Cin, skip, Cb, dW, db, D, B);
+  if (Cout == 16) wgrad_launch<1>(ctx, dout, Cout, in, Cin, skip, Cb, dW, db, D, B);
+  else wgrad_launch<2>(ctx, dout, Cout, in, Cin, skip, Cb, dW, db, D, B);
 }
 
 // After a synchronisation: a bounded wait that expired in a tcgen05
@@ -966,7 +962,7 @@ void backward(cmg_unet *U, int B, const Fields &F) {
     const LayerSpec &L = kLayers[l];
     const int D = dim_of(U, L.lvl);
     float *gw = U->grads + layer_offset(l);
-    wgrad(U, g, L.cout, in, L.cin, skip, Cb, gw, gw + (int64_t)L.cout * 27 * L.cin, D, B);
+    wgrad(U->ctx, g, L.cout, in, L.cin, skip, Cb, gw, gw + (int64_t)L.cout * 27 * L.cin, D, B);
     if (gin) conv(U, l, g, L.cout, nullptr, below, gin, L.cin, D, B, false);
   };
   // decoder level 0
@@ -1285,6 +1281,22 @@ int cmg_unet_grad_clip_stats(cmg_unet *U, double *last_norm, double *mean_norm, 
     if (mean_norm) *mean_norm = h[1];
     if (steps) *steps = (int64_t)h[2];
     if (clipped) *clipped = (int64_t)h[4];
+    return (int)CMG_OK;
+  });
+}
+
+int cmg_debug_conv_wgrad(cmg_ctx *ctx, const uint16_t *dout, int cout, const uint16_t *in, int cin,
+                         const uint16_t *skip, int skip_channels, int grid_dim, int batch, float *dw, float *db) {
+  return unet_guard([&] {
+    if (!ctx || !dout || !in || !dw || !db || grid_dim < 4 || grid_dim % 4 || batch < 1) return (int)CMG_ERR_INVALID_ARG;
+    if ((cout != 16 && cout != 32 && cout != 64) || cin < 16 || cin > 96 || cin % 16) return (int)CMG_ERR_INVALID_ARG;
+    if (skip ? skip_channels < 16 || skip_channels % 16 || skip_channels >= cin : skip_channels != 0)
+      return (int)CMG_ERR_INVALID_ARG;
+    cudaSetDevice(ctx->device);
+    CMG_CUDA(cudaMemsetAsync(dw, 0, sizeof(float) * cout * 27 * cin, ctx->stream));
+    CMG_CUDA(cudaMemsetAsync(db, 0, sizeof(float) * cout, ctx->stream));
+    auto b16 = [](const uint16_t *p) { return reinterpret_cast<const __nv_bfloat16 *>(p); };
+    cmg::wgrad(ctx, b16(dout), cout, b16(in), cin, b16(skip), skip_channels, dw, db, grid_dim, batch);
     return (int)CMG_OK;
   });
 }
