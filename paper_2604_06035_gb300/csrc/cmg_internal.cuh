@@ -386,6 +386,10 @@ namespace cmg {
 
 constexpr int kThreads = 256;
 
+// Largest level whose FP64 kernels run one thread per cell (launch.cu, pcg.cu):
+// 4 n threads fill the 152 SMs about once.
+constexpr int64_t kCellOcts = 40000;
+
 inline unsigned blocks_for(int64_t n, int t = kThreads) { return (unsigned)((n + t - 1) / t); }
 
 // Launch with programmatic dependent launch allowed: the next kernel on the

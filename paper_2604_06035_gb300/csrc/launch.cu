@@ -14,12 +14,15 @@ namespace cmg {
 // issue once per ~64 clocks and sub-partition), so that a launch which does
 // not fill the GPU ends sooner; above, the per-cell loads and index reads
 // cost more.  Residuals and prolongations: up to where 4 n threads fill the
-// 152 SMs about once; colour passes gain further.  Measured (GB300, per
-// solve): 32^3 0.959 -> 0.873 ms, 64^3 two-level CG 2.34 -> 2.27 ms; 128^3
-// two-level 4.13 -> 4.06 ms with passes per cell up to its 179k-oct level,
-// 4.16 ms with its residuals and prolongations too, 4.62 ms with everything
-// on the 262k-oct level.
-constexpr int64_t kCellOcts = 40000, kCellSweepOcts = 200000;
+// 152 SMs about once (kCellOcts); colour passes gain further.  Measured
+// (GB300, per solve): 32^3 0.959 -> 0.873 ms, 64^3 two-level CG 2.34 -> 2.27
+// ms; 128^3 two-level 4.13 -> 4.06 ms with passes per cell up to its 179k-oct
+// level, 4.16 ms with its residuals and prolongations too, 4.62 ms with
+// everything on the 262k-oct level.  Passes per cell up to 40k / 200k octs on a
+// refined level of 73k octs 1.041 / 0.957 ms, 100k 1.274 / 1.131, 126k 1.452 /
+// 1.426, 162k 1.475 / 1.421, 192k 1.765 / 1.681; at 214k the level's own passes
+// take the same either way.
+constexpr int64_t kCellSweepOcts = 200000;
 
 // ------------------------------------------------------------ launchers
 // Algorithmic work per launch (for the profile): bytes are the minimum
@@ -111,9 +114,9 @@ void resid_restrict(cmg_level *L, int m, bool restrict_to_coarse, bool norm, boo
         done = true;
       }
     }
-    if (done)
-      ;
-    else if (restrict_to_coarse && !norm && !emit_scale && c1_swept)
+    if (done) {
+      // launched above
+    } else if (restrict_to_coarse && !norm && !emit_scale && c1_swept)
       launch_k(k_resid<T, false, true, false, false, false, true>, nb, kThreads, s,
           g.nbr, phi_of<T>(g), g_of<T>(g), act, g.n, g.n_alloc, g.father, cg, cphi, cn, cna, zero_coarse_phi,
           nullptr, nullptr, nullptr, nullptr, 0.0);
@@ -321,7 +324,8 @@ void set_density(cmg_level *L, const double *rho, double rho_bar, double four_pi
   if (g.n == 0) return;
   const double scale = -g.h * g.h / 6.0 * four_pi_g;
   LaunchScope ls(L->ctx, K_CONVERT, g.n * 8.0 * 16.0, g.n * 16.0);
-  (wide(rho) ? k_set_density<true> : k_set_density<false>)<<<blocks_for(g.n), kThreads, 0, L->ctx->stream>>>(rho, g.n, rho_bar, scale, g.g);
+  const auto kernel = wide(rho) ? k_set_density<true> : k_set_density<false>;
+  kernel<<<blocks_for(g.n), kThreads, 0, L->ctx->stream>>>(rho, g.n, rho_bar, scale, g.g);
   CMG_CUDA(cudaGetLastError());
 }
 
@@ -344,9 +348,11 @@ void pack_field(cmg_level *L, int m, int field, int prec, const void *in) {
   const unsigned nb = blocks_for(g.n);
   LaunchScope ls(L->ctx, K_CONVERT, g.n * 8.0 * 2.0 * (prec == CMG_PREC_FP64 ? 8.0 : 4.0), 0.0);
   if (prec == CMG_PREC_FP64)
-    launch_k(wide(in) ? k_pack<true, double> : k_pack<false, double>, nb, kThreads, s, (const double *)in, g.n, stride, scale, field == 0 ? g.phi : g.g);
+    launch_k(wide(in) ? k_pack<true, double> : k_pack<false, double>, nb, kThreads, s, (const double *)in, g.n, stride,
+             scale, field == 0 ? g.phi : g.g);
   else
-    launch_k(wide(in) ? k_pack<true, float> : k_pack<false, float>, nb, kThreads, s, (const float *)in, g.n, stride, scale, field == 0 ? g.phi32 : g.g32);
+    launch_k(wide(in) ? k_pack<true, float> : k_pack<false, float>, nb, kThreads, s, (const float *)in, g.n, stride,
+             scale, field == 0 ? g.phi32 : g.g32);
   CMG_CUDA(cudaGetLastError());
 }
 
@@ -359,9 +365,11 @@ void unpack_field(cmg_level *L, int m, int field, int prec, void *out) {
   const unsigned nb = blocks_for(g.n);
   LaunchScope ls(L->ctx, K_CONVERT, g.n * 8.0 * 2.0 * (prec == CMG_PREC_FP64 ? 8.0 : 4.0), 0.0);
   if (prec == CMG_PREC_FP64)
-    launch_k(wide(out) ? k_unpack<true, double> : k_unpack<false, double>, nb, kThreads, s, field == 0 ? g.phi : g.g, g.n, stride, scale, (double *)out);
+    launch_k(wide(out) ? k_unpack<true, double> : k_unpack<false, double>, nb, kThreads, s, field == 0 ? g.phi : g.g,
+             g.n, stride, scale, (double *)out);
   else
-    launch_k(wide(out) ? k_unpack<true, float> : k_unpack<false, float>, nb, kThreads, s, field == 0 ? g.phi32 : g.g32, g.n, stride, scale, (float *)out);
+    launch_k(wide(out) ? k_unpack<true, float> : k_unpack<false, float>, nb, kThreads, s, field == 0 ? g.phi32 : g.g32,
+             g.n, stride, scale, (float *)out);
   CMG_CUDA(cudaGetLastError());
 }
 

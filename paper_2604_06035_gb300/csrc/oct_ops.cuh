@@ -340,13 +340,6 @@ __device__ __forceinline__ void sweep_cell_run(int64_t i, int q, const CellRun &
   dst[i * 4 + q] = out;
 }
 
-// Residual of oct i: d = fma(s, 1/6, g) - phi per cell, r = (-6 / h^2) d.
-// Returns the sum of d^2 over the oct (NORM; accumulated in FP64 for FP64
-// data, in FP32 within the oct for FP32 data, whose FP64 conversions would
-// otherwise bind the kernel to GB300's FP64 pipe).  RESTRICT: a fully active oct
-// writes its father cell g_c = 0.5 * sum_8 d (= -h_c^2/6 * mean_8 r) and, if
-// zero_cphi, zeroes the father's phi.  EMIT: g32 = (float)(d * inv_s).
-// ROUT: r oct-major.  ZPHI: phi taken as zero on real octs.
 // The FP32 right-hand side of a mixed-precision solve's correction problem,
 // (float)(x * s) with s a power of two: the scaling and the rounding to FP32
 // (to nearest, ties to even) formed in integer operations, since GB300
@@ -407,6 +400,13 @@ __device__ __forceinline__ ResidIdx resid_idx(int64_t i, const int32_t *__restri
   return x;
 }
 
+// Residual of oct i: d = fma(s, 1/6, g) - phi per cell, r = (-6 / h^2) d.
+// Returns the sum of d^2 over the oct (NORM; accumulated in FP64 for FP64
+// data, in FP32 within the oct for FP32 data, whose FP64 conversions would
+// otherwise bind the kernel to GB300's FP64 pipe).  RESTRICT: a fully active oct
+// writes its father cell g_c = 0.5 * sum_8 d (= -h_c^2/6 * mean_8 r) and, if
+// zero_cphi, zeroes the father's phi.  EMIT: g32 = (float)(d * inv_s).
+// ROUT: r oct-major.  ZPHI: phi taken as zero on real octs.
 //
 // C1Z: the last operation on this level was a colour-1 pass over every oct
 // with the colour-0 values, g and ghost values the residual now reads.  That
@@ -446,7 +446,7 @@ __device__ __forceinline__ double resid_oct_idx(int64_t i, const ResidIdx &x, co
   double acc = 0.0;
   if constexpr (ZPHI && NORM && !RESTRICT && !EMIT && !ROUT) {
     // phi taken as zero: away from the Dirichlet ghosts every sum is zero and
-    // fma(0, 1/6, g) = g (256^3 level: 118 -> 45 us)
+    // fma(0, 1/6, g) = g (256^3 level, cold cache: 118 -> 59 us)
     if (max(max(max(nb[0], nb[1]), max(nb[2], nb[3])), max(nb[4], nb[5])) < n && m == 0xFFu) {
 #pragma unroll
       for (int p = 0; p < 2; ++p)

@@ -58,8 +58,6 @@ __device__ __forceinline__ void block_partial(double v, double *part) {
 // instructions and 112 loads; now 8, then 16 with the neighbours summed in
 // integers, for 192 bytes more traffic.
 constexpr int kPlaneThreads = 2 * kPcgThreads, kCellThreads4 = 4 * kPcgThreads;
-// largest level that runs four threads per oct (as the other FP64 kernels)
-constexpr int64_t kPcgCellOcts = 40000;
 
 // r = g + nbsum(phi) / 6 - phi (phi's ghost octs hold the Dirichlet values),
 // in place in the right-hand side array g (plane stride 4 n), which holds r
@@ -401,7 +399,7 @@ void pcg_body(cmg_level *L, const cmg_solve_params *p, int64_t *updates) {
   }
   {
     LaunchScope ls(L->ctx, K_RESID64, 8.0 * v.n * 16.0 + 24.0 * v.n, 8.0 * v.n * 9.0);
-    const bool cells = v.n <= kPcgCellOcts;
+    const bool cells = v.n <= kCellOcts;
     launch_k(cells ? k_pcg_apply_cell : k_pcg_apply, v.nb, cells ? kCellThreads4 : kPcgThreads, s, g.nbr, v.p, v.n, v.na,
              v.q, v.part);
   }

@@ -295,7 +295,8 @@ void segment_post(cmg_level *L, const cmg_solve_params *p) {
   if (p->krylov == 1) pcg_post(L);
   {
     LaunchScope ls(L->ctx, K_CONVERT, 0.0, 0.0);
-    k_zero_if<<<std::min(blocks_for(8 * g.n), (unsigned)L->ctx->num_sms), kThreads, 0, L->ctx->stream>>>(ctrl_dev(L), g.phi, g.n, g.n_alloc);
+    const unsigned nb = std::min(blocks_for(8 * g.n), (unsigned)L->ctx->num_sms);
+    k_zero_if<<<nb, kThreads, 0, L->ctx->stream>>>(ctrl_dev(L), g.phi, g.n, g.n_alloc);
     CMG_CUDA(cudaGetLastError());
   }
   if (L->periodic_full) subtract_mean(L);

@@ -1,19 +1,19 @@
 // tail.cu -- the small multigrid levels of a V-cycle in one launch.
 //
 // Small levels' work does not fill the GPU and each operation would cost a
-// full kernel launch.  The tail kernel runs every
-// operation of the V-cycle from MG level m0 down to the coarsest and back up:
-// pre-smoothing, residual + restriction, the coarsest solve (exact 2^3
-// transform or red-black sweeps), prolongation and post-smoothing.
+// full kernel launch.  The tail kernel runs every operation of the V-cycle from
+// MG level m0 down to the coarsest and back up: pre-smoothing, residual +
+// restriction, the coarsest solve (exact 2^3 transform or red-black sweeps),
+// prolongation and post-smoothing.
 //   * Grid tail: one cooperative launch of one CTA per SM.  A level's octs
 //     are split into one contiguous chunk per CTA; operations are separated
 //     by a grid barrier (a word in the solve's control block, bounded waits
-//     that record CMG_ERR_TIMEOUT); loads go through L2
-//     (ld.global.cg), since another CTA may have written the data.  Levels
-//     small enough for one SM run inside the same launch on CTA 0 alone,
-//     with block barriers, while the others wait at the next grid barrier.
-//   * Single-CTA tail: when even the first tail level fits one SM, one CTA of 512 or
-//     1024 threads with block barriers and L1 loads.
+//     that record CMG_ERR_TIMEOUT), whose release and acquire let plain loads
+//     see what other CTAs wrote.  Levels small enough for one SM run inside
+//     the same launch on CTA 0 alone, with block barriers, while the others
+//     wait at the next grid barrier.
+//   * Single-CTA tail: when even the first tail level fits one SM, one CTA of
+//     512 (FP64) or 1024 threads with block barriers.
 // The arithmetic is the same per-oct code as the one-launch-per-operation
 // path (oct_ops.cuh), so every schedule gives the same results.
 #include "cmg_internal.cuh"

@@ -8,13 +8,15 @@
 // [Cin][27][Cout] for the input gradient, tap t = 9 (dz+1) + 3 (dy+1) + (dx+1);
 // master parameters, gradients and Adam moments are FP32.
 //
-// Convolutions are implicit GEMMs on mma.sync m16n8k16 (bf16 in, fp32
-// accumulate).  A block owns a 4x4x4 voxel brick: per 16-channel slice it
-// stages the brick's 6x6x6 periodic halo (216 rows of 32 B) and the 27 taps of
-// the weight slice in shared memory, and every tap's A fragment is an ldmatrix
-// of halo rows shifted by the tap offset -- each input value is read from
-// global memory once per slice instead of 27 times.  The weight gradient uses
-// the same halo with ldmatrix.trans fragments and reduces over bricks.
+// Convolutions and input gradients on grids of a multiple of 16 run on the
+// tcgen05 kernels of conv_tc.cuh.  Below that (or on request) they are implicit
+// GEMMs on mma.sync m16n8k16 (bf16 in, fp32 accumulate): a block owns a 4x4x4
+// voxel brick, per 16-channel slice it stages the brick's 6x6x6 periodic halo
+// (216 rows of 32 B) and the 27 taps of the weight slice in shared memory, and
+// every tap's A fragment is an ldmatrix of halo rows shifted by the tap offset
+// -- each input value is read from global memory once per slice instead of 27
+// times.  The weight gradient (k_conv_wgrad) stages the same bricks, in another
+// layout, and sums over runs of them.
 #include <cuda_bf16.h>
 
 #include <cmath>
